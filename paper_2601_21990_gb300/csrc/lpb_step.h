@@ -212,6 +212,7 @@ __device__ __forceinline__ void gather_round(const int (&c)[Round<T, G>::K], con
     }
 }
 
+// acc += the row's entries [beg, end), a round at a time
 template <typename T, int V, int G>
 __device__ __forceinline__ void gather_range(const int* __restrict__ ci, const T* __restrict__ va,
                                              const T* __restrict__ src, int ld, int colg, int beg, int end,
@@ -444,21 +445,6 @@ __device__ __forceinline__ void step_body(const StepArgs<T>& a, const int bx, co
             if (std::is_same<T, dfloat>::value) P.isigma[q] = T(1) / P.sigma[q];
         }
     }
-    __syncthreads();
-    // Programmatic dependent launch: everything above reads only data that
-    // the previous kernel does not write (per-column parameters, Halpern
-    // weights).  That holds because only step kernels after an interval's
-    // first are launched as programmatic dependents, and their predecessor
-    // is a step kernel; the first primal step of an interval follows the
-    // check, admission, extraction, compaction and migration kernels that do
-    // write those parameters, and is launched without the attribute
-    // (launch_iteration).  Wait for the predecessor to complete before
-    // touching the iterates, then let the next step kernel start its own
-    // prologue on the SMs this grid frees.
-    if (a.pdl) {
-        asm volatile("griddepcontrol.wait;" ::: "memory");
-        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    }
     // one restart group in the whole batch: its Halpern weights as scalars
     // (the primal step takes the previous iteration's, the dual step this one's)
     const int hu = a.uni >= 0 ? 2 * (a.uni * (a.ce + 1) + a.t + (PRIMAL ? 0 : 1)) : 0;
@@ -468,22 +454,58 @@ __device__ __forceinline__ void step_body(const StepArgs<T>& a, const int bx, co
     const int colg = active ? col0 : tile0;
     const unsigned gmask = G == 32 ? 0xffffffffu : (((1u << G) - 1u) << ((threadIdx.x & 31) & ~(G - 1)));
 
-    if (bx < a.n_lblocks) {
-        const int li = a.lseg[2 * bx], sg = a.lseg[2 * bx + 1];
-        const int s0 = a.lseg0[li], ns = a.lseg0[li + 1] - s0;
+    // The block's first entries: of its segment's piece, or of its row
+    // group's first row.
+    const bool is_seg = bx < a.n_lblocks;
+    const int stride = (gx - a.n_lblocks) * GPB;
+    int r = (bx - a.n_lblocks) * GPB + grp;
+    int beg = 0, end = 0;
+    int c[K];
+    T av[K];
+    if (is_seg) {
+        const int li = a.lseg[2 * bx], sg = a.lseg[2 * bx + 1], ns = a.lseg0[li + 1] - a.lseg0[li];
         const int row = a.long_rows[li];
         const int rb0 = a.rp[row], re0 = a.rp[row + 1];
         const int sl = (re0 - rb0 + ns - 1) / ns;  // entries per segment
         const int rb = min(re0, rb0 + sg * sl), re = min(re0, rb + sl);
         const int piece = (re - rb + GPB - 1) / GPB;
-        const int beg = min(re, rb + grp * piece), end = min(re, beg + piece);
+        beg = min(re, rb + grp * piece);
+        end = min(re, beg + piece);
+        load_round<T, G>(a.ci, a.va, beg, end, c, av);
+    } else if (r < a.rows) {
+        beg = a.rp[r];
+        end = a.rp[r + 1];
+        load_round<T, G>(a.ci, a.va, beg, end - beg <= a.long_thr ? end : beg, c, av);
+    }
+    __syncthreads();
+    // Programmatic dependent launch: everything above reads only data that
+    // the previous kernel does not write (the matrix, per-column parameters,
+    // Halpern weights), so its round trips overlap the end of that kernel: a
+    // step then waits for its gathers alone.  That holds because only step
+    // kernels after an interval's first are launched as programmatic
+    // dependents, and their predecessor is a step kernel; the first primal
+    // step of an interval follows the check, admission, extraction,
+    // compaction and migration kernels that do write those parameters, and is
+    // launched without the attribute (launch_iteration).  Wait for the
+    // predecessor to complete before touching the iterates, then let the next
+    // step kernel start its own prologue on the SMs this grid frees.
+    if (a.pdl) {
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    }
+
+    if (is_seg) {
         T acc[V];
 #pragma unroll
         for (int v = 0; v < V; ++v) acc[v] = T(0);
-        gather_range<T, V, G>(a.ci, a.va, a.src, a.ld, colg, beg, end, gmask, acc);
+        gather_round<T, V, G>(c, av, min(R, end - beg), a.src, a.ld, colg, gmask, acc);
+        if (end - beg > R) gather_range<T, V, G>(a.ci, a.va, a.src, a.ld, colg, beg + R, end, gmask, acc);
         fin<V>(acc);
         if (!long_row_reduce<T, V, G>(acc, red)) return;
         // only row group 0 (lanes 0 .. G-1 of warp 0) continues
+        const int li = a.lseg[2 * bx], sg = a.lseg[2 * bx + 1];
+        const int s0 = a.lseg0[li], ns = a.lseg0[li + 1] - s0;
+        const int row = a.long_rows[li];
         if (ns > 1) {
             if (active) stv_cg(a.part + (size_t)(s0 + sg) * a.ld + col0, acc);
             __threadfence();
@@ -513,16 +535,6 @@ __device__ __forceinline__ void step_body(const StepArgs<T>& a, const int bx, co
         return;
     }
 
-    const int stride = (gx - a.n_lblocks) * GPB;
-    int r = (bx - a.n_lblocks) * GPB + grp;
-    int beg = 0, end = 0;
-    int c[K];
-    T av[K];
-    if (r < a.rows) {
-        beg = a.rp[r];
-        end = a.rp[r + 1];
-        load_round<T, G>(a.ci, a.va, beg, end - beg <= a.long_thr ? end : beg, c, av);
-    }
 #pragma unroll 1
     while (r < a.rows) {
         const int rn = r + stride;
