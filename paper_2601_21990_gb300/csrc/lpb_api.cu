@@ -424,12 +424,33 @@ lpb_err time_steps_any(lpb_ctx* h, int count, int R, double* up, double* ud) {
                                          : time_steps<double>(h, count, R, up, ud);
 }
 
+// the packed short rows of A~ or A~^T in the iterate types that the handle's
+// solves may run in
+lpb_err pack_rows(lpb_ctx* h, Csr& c) {
+    const bool at = &c == &h->At, mixed = h->opt.precision == LPB_MIXED;
+    RowVectors<float> v32{};
+    RowVectors<double> v64{};
+    RowVectors<dfloat> vdf{};
+    if (mixed)
+        v32 = at ? RowVectors<float>{c.v32, h->cs32, h->xls32, h->xus32}
+                 : RowVectors<float>{c.v32, nullptr, h->ls32, h->us32};
+    if (!mixed || (polish_enabled(h) && !polish_dfloat(h)))
+        v64 = at ? RowVectors<double>{c.v64, h->cs, h->xls, h->xus} : RowVectors<double>{c.v64, nullptr, h->ls, h->us};
+    if (polish_dfloat(h))
+        vdf = at ? RowVectors<dfloat>{h->at_dfl, h->cs_dfl, h->xls_dfl, h->xus_dfl}
+                 : RowVectors<dfloat>{h->a_dfl, nullptr, h->ls_dfl, h->us_dfl};
+    CU(build_short_rows(c, v32, v64, vdf, h->stream));
+    return LPB_OK;
+}
+
 lpb_err apply_shape(lpb_ctx* h, Csr& c, int thr, int shift) {
     if (c.long_thr != thr) {
         c.long_thr = thr;
         CU(build_long_rows(c, h->stream));
+        lpb_err rc = pack_rows(h, c);
+        if (rc != LPB_OK) return rc;
         // the segment scratch follows the new long-row lists
-        lpb_err rc = ensure_long_scratch(h, std::max(h->lr_cap, h->ws_cap), true);
+        rc = ensure_long_scratch(h, std::max(h->lr_cap, h->ws_cap), true);
         if (rc != LPB_OK) return rc;
     }
     c.g_shift = shift;
@@ -701,6 +722,10 @@ lpb_err lpb_create(int32_t m, int32_t n, int64_t nnz, const int64_t* row_ptr, co
             CU(split_df(h->xus, (df*)h->xus_dfl, n, false, s));
             CU(split_df(h->ls, (df*)h->ls_dfl, m, false, s));
             CU(split_df(h->us, (df*)h->us_dfl, m, false, s));
+        }
+        for (Csr* c : {&h->A, &h->At}) {
+            const lpb_err rc = pack_rows(h, *c);
+            if (rc != LPB_OK) return rc;
         }
         // ||c~||, ||b~|| (w0) and the power iteration (eta)
         double* scal = nullptr;
@@ -997,6 +1022,8 @@ void lpb_destroy(lpb_handle h) {
     free_list(h->fixed_allocs);
     free_long_rows(h->A);
     free_long_rows(h->At);
+    free_short_rows(h->A);
+    free_short_rows(h->At);
     free_long_scratch(h);
     if (h->own_stream && h->stream) cudaStreamDestroy(h->stream);
     delete h;

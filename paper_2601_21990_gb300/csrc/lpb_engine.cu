@@ -41,6 +41,10 @@ IterData<T> iter_data(const lpb_ctx* h, const Lane& ln) {
     d.At = h->At;
     d.a_vals = pick<T>(h->A.v64, h->A.v32, h->a_dfl);
     d.at_vals = pick<T>(h->At.v64, h->At.v32, h->at_dfl);
+    d.a_pv = pick<T>(h->A.pv64, h->A.pv32, h->A.pvdf);
+    d.a_pk = pick<T>(h->A.pk64, h->A.pk32, h->A.pkdf);
+    d.at_pv = pick<T>(h->At.pv64, h->At.pv32, h->At.pvdf);
+    d.at_pk = pick<T>(h->At.pk64, h->At.pk32, h->At.pkdf);
     d.c = pick<T>(h->cs, h->cs32, h->cs_dfl);
     d.xl = pick<T>(h->xls, h->xls32, h->xls_dfl);
     d.xu = pick<T>(h->xus, h->xus32, h->xus_dfl);

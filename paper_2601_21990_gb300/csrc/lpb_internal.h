@@ -66,6 +66,18 @@ struct Csr {
     float* v32lo = nullptr;     // v64 - v32 rounded to FP32: (v32, v32lo) is v64 in double-float
     int* long_rows = nullptr;   // rows with > long_thr entries
     int n_long = 0;
+    // The other rows as the step kernels take them (build_short_rows): in
+    // windows sorted by length, each row's entries together, from a multiple of
+    // four on, and its cost and bounds beside its record.
+    int4* srec = nullptr;       // row, its first four entries (entry index / 4), pairs of entries, entries
+    int n_short = 0;
+    int* pci = nullptr;         // entries: columns, and values in the iterate types in use
+    float* pv32 = nullptr;
+    double* pv64 = nullptr;
+    dfloat* pvdf = nullptr;
+    float* pk32 = nullptr;      // per record: cost (A~^T), lower and upper bound, 0
+    double* pk64 = nullptr;
+    dfloat* pkdf = nullptr;
     int long_thr = kLongRow;    // rows longer than this get a whole block (tunable)
     int g_shift = 0;            // step kernels use (lanes per row from the batch width) >> g_shift
     // Step kernels cut a long row into segments of at most kStepSeg entries,
@@ -171,6 +183,16 @@ cudaError_t exclusive_scan_i32(const int* in, int* out, int count, int* total_de
 // a.long_thr (frees an old list); free_long_rows releases them
 cudaError_t build_long_rows(Csr& a, cudaStream_t s);
 void free_long_rows(Csr& a);
+// (re)builds the packed short rows for the rows that build_long_rows left
+// out, with the values and row vectors of the iterate types whose values are
+// given (c null: no costs); free_short_rows releases them
+template <typename T>
+struct RowVectors {
+    const T *vals, *c, *lo, *hi;
+};
+cudaError_t build_short_rows(Csr& a, RowVectors<float> v32, RowVectors<double> v64, RowVectors<dfloat> vdf,
+                             cudaStream_t s);
+void free_short_rows(Csr& a);
 cudaError_t ruiz_pock_chambolle(const Csr& a, const double* a_vals, const Csr& at, const double* at_vals,
                                 int ruiz_iters, int pock_chambolle, double* d_r, double* d_c,
                                 double* tmp_r, double* tmp_c, cudaStream_t s);
@@ -205,6 +227,8 @@ struct IterData {
     Csr A, At;                 // scaled CSRs (values in T taken from v64 / v32)
     const T* a_vals;
     const T* at_vals;
+    const T *a_pv, *a_pk;      // packed short rows' values and row vectors
+    const T *at_pv, *at_pk;
     const T *c, *xl, *xu;      // scaled base vectors (n)
     const T *l, *u;            // scaled row bounds (m)
     ColParams<T> col;

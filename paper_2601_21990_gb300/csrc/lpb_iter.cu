@@ -37,29 +37,42 @@ namespace lpb {
 
 namespace {
 
-template <typename T, int G, bool CHECK, bool PRIMAL>
-__global__ void __launch_bounds__(kBlock, (MinBlocks<T, G, PRIMAL>::v)) k_step(const __grid_constant__ StepArgs<T> a) {
-    step_body<T, G, CHECK, PRIMAL>(a, (int)blockIdx.x, (int)blockIdx.y, (int)gridDim.x);
+template <typename T, int G, int B, bool CHECK, bool PRIMAL>
+__global__ void __launch_bounds__(kBlock, (MinBlocks<T, G, B>::v)) k_step(const __grid_constant__ StepArgs<T> a) {
+    step_body<T, G, B, CHECK, PRIMAL>(a, (int)blockIdx.x, (int)blockIdx.y, (int)gridDim.x);
 }
 
-template <typename T, int G, bool CHECK, bool PRIMAL>
-cudaError_t launch_k(const StepArgs<T>& a, cudaStream_t s) {
+// The step with B gathers at a time; with `if_fits`, only when its blocks
+// are all resident at once (*fits).
+template <typename T, int G, int B, bool CHECK, bool PRIMAL>
+cudaError_t launch_k(const StepArgs<T>& a, bool if_fits, bool* fits, cudaStream_t s) {
     constexpr int V = Vec<T>::V, GPB = kBlock / G, TN = G * V;
     static std::atomic<int> shape[kShapeDevices];  // static storage: starts at 0
     int sms = 0, per_sm = 0;
-    const cudaError_t e = launch_shape(shape, k_step<T, G, CHECK, PRIMAL>, &sms, &per_sm);
+    const cudaError_t e = launch_shape(shape, k_step<T, G, B, CHECK, PRIMAL>, &sms, &per_sm);
     if (e != cudaSuccess) return e;
-    const int need = (a.rows + GPB - 1) / GPB;
+    const int need = (a.n_short + GPB - 1) / GPB, tiles = (a.ncol + TN - 1) / TN;
+    *fits = ((long long)a.n_lblocks + need) * tiles <= (long long)sms * per_sm;
+    if (if_fits && !*fits) return cudaSuccess;
     const int persist = need < sms * per_sm ? need : sms * per_sm;
-    const dim3 grid(a.n_lblocks + persist, (a.ncol + TN - 1) / TN);
-    return launch_with(k_step<T, G, CHECK, PRIMAL>, grid, a, a.pdl != 0, s);
+    return launch_with(k_step<T, G, B, CHECK, PRIMAL>, dim3(a.n_lblocks + persist, tiles), a, a.pdl != 0, s);
+}
+
+template <typename T, int G, bool CHECK, bool PRIMAL>
+cudaError_t launch_depth(const StepArgs<T>& a, cudaStream_t s) {
+    bool fits = false;
+    if constexpr (kDeep<G> > 0) {
+        const cudaError_t e = launch_k<T, G, kDeep<G>, CHECK, PRIMAL>(a, true, &fits, s);
+        if (e != cudaSuccess || fits) return e;
+    }
+    return launch_k<T, G, kFlat, CHECK, PRIMAL>(a, false, &fits, s);
 }
 
 template <typename T, int G>
 cudaError_t launch_step(bool primal, bool check, const StepArgs<T>& a, cudaStream_t s) {
     if (a.rows == 0 || a.ncol == 0) return cudaSuccess;
-    if (primal) return check ? launch_k<T, G, true, true>(a, s) : launch_k<T, G, false, true>(a, s);
-    return check ? launch_k<T, G, true, false>(a, s) : launch_k<T, G, false, false>(a, s);
+    if (primal) return check ? launch_depth<T, G, true, true>(a, s) : launch_depth<T, G, false, true>(a, s);
+    return check ? launch_depth<T, G, true, false>(a, s) : launch_depth<T, G, false, false>(a, s);
 }
 
 template <typename T>

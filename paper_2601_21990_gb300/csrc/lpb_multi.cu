@@ -16,16 +16,8 @@
 #include "lpb_joint_grid.h"
 #include "lpb_step.h"
 
-// resident blocks per SM of the joint kernels with row groups of 8 or more
-// lanes, FP32 and FP64 (see MultiMinBlocks)
-#ifndef LPB_MULTI_MIN_BLOCKS_F32
-#define LPB_MULTI_MIN_BLOCKS_F32 8
-#endif
-#ifndef LPB_MULTI_MIN_BLOCKS_F64
-#define LPB_MULTI_MIN_BLOCKS_F64 7
-#endif
-// the double-float joint kernels (the joint polish phase): one block fewer
-// than the single kernels, whose 72 registers the part lookup would overflow
+// the double-float joint kernels: one block fewer than the single kernels,
+// whose 72 registers the part lookup would overflow
 #ifndef LPB_MULTI_MIN_BLOCKS_DF
 #define LPB_MULTI_MIN_BLOCKS_DF 6
 #endif
@@ -48,25 +40,20 @@ struct MultiStepArgs {
 // kernel parameters stay within the classic 4 KB limit
 static_assert(sizeof(MultiStepArgs<double>) <= 4096, "joint step arguments exceed 4 KB");
 
-// Resident blocks per SM of the joint kernels: those the single-matrix
-// kernels reach with their register counts (the part lookup and the
-// indexed arguments cost the joint kernels a few registers more).  Row
-// groups of 4 lanes or fewer keep the single kernels' bound, where the
-// tighter cap would spill.
-template <typename T, int G, bool PRIMAL> struct MultiMinBlocks {
-    static constexpr int cap = G <= 4 ? 5 : std::is_same<T, float>::value ? LPB_MULTI_MIN_BLOCKS_F32
-                                                                           : LPB_MULTI_MIN_BLOCKS_F64;
-    static constexpr int v = MinBlocks<T, G, PRIMAL>::v > cap ? MinBlocks<T, G, PRIMAL>::v : cap;
-};
-template <int G, bool PRIMAL> struct MultiMinBlocks<dfloat, G, PRIMAL> {
-    static constexpr int v = LPB_MULTI_MIN_BLOCKS_DF;
+// Resident blocks per SM of the joint kernels: the single-matrix kernels'
+// (the part lookup and the indexed arguments cost a few registers more).
+template <typename T, int G, int B> struct MultiMinBlocks {
+    static constexpr int one = MinBlocks<T, G, B>::v;
+    static constexpr int v = std::is_same<T, dfloat>::value && one > LPB_MULTI_MIN_BLOCKS_DF ? LPB_MULTI_MIN_BLOCKS_DF
+                             : one > 8                                                         ? 8
+                                                                                               : one;
 };
 
-template <typename T, int G, bool CHECK, bool PRIMAL>
-__global__ void __launch_bounds__(kBlock, (MultiMinBlocks<T, G, PRIMAL>::v))
+template <typename T, int G, int B, bool CHECK, bool PRIMAL>
+__global__ void __launch_bounds__(kBlock, (MultiMinBlocks<T, G, B>::v))
     k_step_multi(const __grid_constant__ MultiStepArgs<T> m) {
     const JointPlace q = joint_place((int)blockIdx.x, m.nparts, m.block0, m.gx);
-    step_body<T, G, CHECK, PRIMAL>(m.part[q.part], q.bx, q.by, q.gx);
+    step_body<T, G, B, CHECK, PRIMAL>(m.part[q.part], q.bx, q.by, q.gx);
 }
 
 // Each part gets the grid k_step would get for it alone: its long-row
@@ -75,31 +62,45 @@ __global__ void __launch_bounds__(kBlock, (MultiMinBlocks<T, G, PRIMAL>::v))
 // SMs idle) come first in the grid, so that their blocks run beside the
 // first wave of the larger parts' blocks.  Which block takes a row does not
 // change the row's arithmetic.
-template <typename T, int G, bool CHECK, bool PRIMAL>
-cudaError_t launch_multi_k(MultiStepArgs<T>& m, bool pdl, cudaStream_t s) {
+// With if_fits, only when all blocks are resident at once (*fits).
+template <typename T, int G, int B, bool CHECK, bool PRIMAL>
+cudaError_t launch_multi_k(MultiStepArgs<T>& m, bool if_fits, bool* fits, bool pdl, cudaStream_t s) {
     constexpr int V = Vec<T>::V, GPB = kBlock / G, TN = G * V;
     static std::atomic<int> shape[kShapeDevices];  // static storage: starts at 0
     int sms = 0, per_sm = 0;
-    const cudaError_t e = launch_shape(shape, k_step_multi<T, G, CHECK, PRIMAL>, &sms, &per_sm);
+    const cudaError_t e = launch_shape(shape, k_step_multi<T, G, B, CHECK, PRIMAL>, &sms, &per_sm);
     if (e != cudaSuccess) return e;
     int nlb[kMaxParts], need[kMaxParts], tiles[kMaxParts];
     for (int p = 0; p < m.nparts; ++p) {
         StepArgs<T>& a = m.part[p];
         a.pdl = pdl ? 1 : 0;
         nlb[p] = a.n_lblocks;
-        need[p] = (a.rows + GPB - 1) / GPB;
+        need[p] = (a.n_short + GPB - 1) / GPB;
         tiles[p] = (a.ncol + TN - 1) / TN;
     }
     const long long total = joint_layout(m.nparts, nlb, need, tiles, sms * per_sm, m.block0, m.gx);
     if (total < 0) return cudaErrorInvalidConfiguration;
-    if (total == 0) return cudaSuccess;
-    return launch_with(k_step_multi<T, G, CHECK, PRIMAL>, dim3((unsigned)total), m, pdl, s);
+    // (a part is cut to a wave of blocks only where it alone exceeds one)
+    *fits = total < (long long)sms * per_sm;
+    if (total == 0 || (if_fits && !*fits)) return cudaSuccess;
+    return launch_with(k_step_multi<T, G, B, CHECK, PRIMAL>, dim3((unsigned)total), m, pdl, s);
+}
+
+template <typename T, int G, bool CHECK, bool PRIMAL>
+cudaError_t launch_multi_depth(MultiStepArgs<T>& m, bool pdl, cudaStream_t s) {
+    bool fits = false;
+    if constexpr (kDeep<G> > 0) {
+        const cudaError_t e = launch_multi_k<T, G, kDeep<G>, CHECK, PRIMAL>(m, true, &fits, pdl, s);
+        if (e != cudaSuccess || fits) return e;
+    }
+    return launch_multi_k<T, G, kFlat, CHECK, PRIMAL>(m, false, &fits, pdl, s);
 }
 
 template <typename T, int G>
 cudaError_t launch_multi_step(bool primal, bool check, MultiStepArgs<T>& m, bool pdl, cudaStream_t s) {
-    if (primal) return check ? launch_multi_k<T, G, true, true>(m, pdl, s) : launch_multi_k<T, G, false, true>(m, pdl, s);
-    return check ? launch_multi_k<T, G, true, false>(m, pdl, s) : launch_multi_k<T, G, false, false>(m, pdl, s);
+    if (primal)
+        return check ? launch_multi_depth<T, G, true, true>(m, pdl, s) : launch_multi_depth<T, G, false, true>(m, pdl, s);
+    return check ? launch_multi_depth<T, G, true, false>(m, pdl, s) : launch_multi_depth<T, G, false, false>(m, pdl, s);
 }
 
 template <typename T>

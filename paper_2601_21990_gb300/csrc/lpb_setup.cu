@@ -209,6 +209,107 @@ __global__ void k_long_scatter(const int* __restrict__ flag, const int* __restri
 }
 
 // ---------------------------------------------------------------------------
+// short rows in the order of the step kernels
+// ---------------------------------------------------------------------------
+// Windows of kWindow rows, each sorted by length, longest first: the row
+// groups of a warp then take rows of about the same length, and rows that lie
+// near one another stay near (a window's rows share what they gather in L2).
+constexpr int kWindow = 2048;
+
+// per window: its rows of at most thr entries
+__global__ void __launch_bounds__(256) k_short_count(const int* __restrict__ rp, int rows, int thr,
+                                                     int* __restrict__ cnt) {
+    __shared__ int sum;
+    if (threadIdx.x == 0) sum = 0;
+    __syncthreads();
+    int mine = 0;
+    for (int q = threadIdx.x; q < kWindow; q += blockDim.x) {
+        const int i = blockIdx.x * kWindow + q;
+        if (i < rows && rp[i + 1] - rp[i] <= thr) ++mine;
+    }
+    if (mine) atomicAdd(&sum, mine);
+    __syncthreads();
+    if (threadIdx.x == 0) cnt[blockIdx.x] = sum;
+}
+
+// one block per window: bitonic sort of (length, place) keys, the rows of
+// more than thr entries last; equal lengths keep their order
+__global__ void __launch_bounds__(1024) k_short_order(const int* __restrict__ rp, int rows, int thr,
+                                                      const int* __restrict__ first, int4* __restrict__ out) {
+    __shared__ unsigned long long key[kWindow];
+    const int base = blockIdx.x * kWindow;
+    for (int q = threadIdx.x; q < kWindow; q += blockDim.x) {
+        const int i = base + q;
+        const int len = i < rows ? rp[i + 1] - rp[i] : INT_MAX;
+        const unsigned desc = len <= thr ? (unsigned)(thr - len) : 0xffffffffu;
+        key[q] = (unsigned long long)desc << 32 | (unsigned)q;
+    }
+    __syncthreads();
+    for (int k = 2; k <= kWindow; k <<= 1)
+        for (int j = k >> 1; j > 0; j >>= 1) {
+            for (int q = threadIdx.x; q < kWindow; q += blockDim.x) {
+                const int p = q ^ j;
+                if (p > q) {
+                    const unsigned long long x = key[q], y = key[p];
+                    if ((x > y) == ((q & k) == 0)) {
+                        key[q] = y;
+                        key[p] = x;
+                    }
+                }
+            }
+            __syncthreads();
+        }
+    for (int q = threadIdx.x; q < kWindow; q += blockDim.x) {
+        if (key[q] >> 32 == 0xffffffffull) continue;
+        const int i = base + (int)(key[q] & 0xffffffffull);
+        out[first[blockIdx.x] + q] = make_int4(i, 0, 0, rp[i + 1] - rp[i]);
+    }
+}
+
+// fours of entries of each record
+__global__ void k_short_fours(const int4* __restrict__ rec, int n, int* __restrict__ cnt) {
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
+        cnt[i] = (rec[i].w + 3) / 4;
+}
+__global__ void k_short_place(int4* __restrict__ rec, int n, const int* __restrict__ first) {
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+        rec[i].y = first[i];
+        rec[i].z = (rec[i].w + 1) / 2;
+    }
+}
+
+// columns of the packed entries, and their values and the rows' vectors: a
+// warp per record; an odd row's last pair is filled up with its last entry's
+// column and the value 0
+__global__ void k_short_cols(const int4* __restrict__ rec, int n, const int* __restrict__ rp,
+                             const int* __restrict__ ci, int* __restrict__ out) {
+    const int warps = gridDim.x * blockDim.x / 32, lane = threadIdx.x & 31;
+    for (int i = (blockIdx.x * blockDim.x + threadIdx.x) / 32; i < n; i += warps) {
+        const int4 r = rec[i];
+        const int b = rp[r.x];
+        for (int e = lane; e < (r.w + 3) / 4 * 4; e += 32)
+            out[(size_t)r.y * 4 + e] = ci[b + (e < r.w ? e : r.w - 1)];
+    }
+}
+template <typename T>
+__global__ void k_short_vals(const int4* __restrict__ rec, int n, const int* __restrict__ rp, RowVectors<T> v,
+                             T* __restrict__ out, T* __restrict__ k) {
+    const int warps = gridDim.x * blockDim.x / 32, lane = threadIdx.x & 31;
+    for (int i = (blockIdx.x * blockDim.x + threadIdx.x) / 32; i < n; i += warps) {
+        const int4 r = rec[i];
+        const int b = rp[r.x];
+        for (int e = lane; e < (r.w + 3) / 4 * 4; e += 32)
+            out[(size_t)r.y * 4 + e] = e < r.w ? v.vals[b + e] : T(0);
+        if (lane == 0) {
+            k[4 * (size_t)i] = v.c ? v.c[r.x] : T(0);
+            k[4 * (size_t)i + 1] = v.lo[r.x];
+            k[4 * (size_t)i + 2] = v.hi[r.x];
+            k[4 * (size_t)i + 3] = T(0);
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------
 // equilibration
 // ---------------------------------------------------------------------------
 // One warp per CSR row: max or sum of |D_r[i] * a * D_c[j]| where, for the
@@ -627,6 +728,83 @@ cudaError_t build_long_rows(Csr& a, cudaStream_t s) {
     }
     if ((e = cudaFreeAsync(flag, s)) != cudaSuccess) return e;
     return build_long_segments(a, s);
+}
+
+void free_short_rows(Csr& a) {
+    if (a.srec) cudaFree(a.srec);  // with all that lies behind it
+    a.srec = nullptr;
+    a.pci = nullptr;
+    a.pv32 = a.pk32 = nullptr;
+    a.pv64 = a.pk64 = nullptr;
+    a.pvdf = a.pkdf = nullptr;
+    a.n_short = 0;
+}
+
+template <typename T>
+static cudaError_t pack_vals(const Csr& a, int n, RowVectors<T> v, T* out, T* k, cudaStream_t s) {
+    if (!v.vals) return cudaSuccess;
+    k_short_vals<T><<<grid_for((long long)n * 32, 256, kStatCap), 256, 0, s>>>(a.srec, n, a.rp, v, out, k);
+    return cudaGetLastError();
+}
+
+cudaError_t build_short_rows(Csr& a, RowVectors<float> v32, RowVectors<double> v64, RowVectors<dfloat> vdf,
+                             cudaStream_t s) {
+    cudaError_t e;
+    if (a.srec && (e = cudaStreamSynchronize(s)) != cudaSuccess) return e;
+    free_short_rows(a);
+    const int n = a.rows - a.n_long;
+    if (n <= 0) return cudaSuccess;
+    // one allocation, for at most three entries a row more than the matrix has
+    const size_t entries = (size_t)a.nnz + 3 * (size_t)n;
+    size_t bytes = 0;
+    auto take = [&](bool wanted, size_t size) {
+        const size_t at = bytes;
+        if (wanted) bytes += (size + 255) / 256 * 256;
+        return at;
+    };
+    const size_t at_rec = take(true, sizeof(int4) * n), at_ci = take(true, 4 * entries);
+    const size_t at_v32 = take(v32.vals, 4 * entries), at_k32 = take(v32.vals, 16 * (size_t)n);
+    const size_t at_v64 = take(v64.vals, 8 * entries), at_k64 = take(v64.vals, 32 * (size_t)n);
+    const size_t at_vdf = take(vdf.vals, 8 * entries), at_kdf = take(vdf.vals, 32 * (size_t)n);
+    char* mem = nullptr;
+    if ((e = cudaMalloc((void**)&mem, bytes)) != cudaSuccess) return e;
+    a.srec = (int4*)(mem + at_rec);
+    a.pci = (int*)(mem + at_ci);
+    if (v32.vals) {
+        a.pv32 = (float*)(mem + at_v32);
+        a.pk32 = (float*)(mem + at_k32);
+    }
+    if (v64.vals) {
+        a.pv64 = (double*)(mem + at_v64);
+        a.pk64 = (double*)(mem + at_k64);
+    }
+    if (vdf.vals) {
+        a.pvdf = (dfloat*)(mem + at_vdf);
+        a.pkdf = (dfloat*)(mem + at_kdf);
+    }
+    const int windows = (a.rows + kWindow - 1) / kWindow;
+    const size_t most = std::max((size_t)windows, (size_t)n);
+    int* cnt = nullptr;
+    if ((e = cudaMallocAsync((void**)&cnt, sizeof(int) * most * 2, s)) != cudaSuccess) return e;
+    int* first = cnt + most;
+    k_short_count<<<windows, 256, 0, s>>>(a.rp, a.rows, a.long_thr, cnt);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if ((e = exclusive_scan_i32(cnt, first, windows, nullptr, s)) != cudaSuccess) return e;
+    k_short_order<<<windows, 1024, 0, s>>>(a.rp, a.rows, a.long_thr, first, a.srec);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    k_short_fours<<<grid_for(n, 256), 256, 0, s>>>(a.srec, n, cnt);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if ((e = exclusive_scan_i32(cnt, first, n, nullptr, s)) != cudaSuccess) return e;
+    k_short_place<<<grid_for(n, 256), 256, 0, s>>>(a.srec, n, first);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if ((e = cudaFreeAsync(cnt, s)) != cudaSuccess) return e;
+    k_short_cols<<<grid_for((long long)n * 32, 256, kStatCap), 256, 0, s>>>(a.srec, n, a.rp, a.ci, a.pci);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if ((e = pack_vals<float>(a, n, v32, a.pv32, a.pk32, s)) != cudaSuccess) return e;
+    if ((e = pack_vals<double>(a, n, v64, a.pv64, a.pk64, s)) != cudaSuccess) return e;
+    if ((e = pack_vals<dfloat>(a, n, vdf, a.pvdf, a.pkdf, s)) != cudaSuccess) return e;
+    a.n_short = n;
+    return cudaSuccess;
 }
 
 cudaError_t ruiz_pock_chambolle(const Csr& a, const double* a_vals, const Csr& at, const double* at_vals,

@@ -10,18 +10,27 @@
 
 #include "lpb_internal.h"
 
-// resident blocks per SM the step kernels are compiled for (register cap)
-#ifndef LPB_STEP_MIN_BLOCKS
-#define LPB_STEP_MIN_BLOCKS 5
+// Resident blocks per SM the step kernels are compiled for (register caps
+// without spills; a spilled byte goes through the same L1 as the gathers, and
+// a few of them per row cost more than a block less).  FP32: the row groups
+// of 32 lanes wait on HBM and gain from every block (10 at 48 registers; on
+// the 1M-row matrix 8 blocks took 140 ms a pass, 10 took 138 ms); the
+// narrower ones run from L2 (8).  Double-float and FP64 hold wider sums.
+#ifndef LPB_STEP_MIN_BLOCKS_WIDE
+#define LPB_STEP_MIN_BLOCKS_WIDE 10
 #endif
-// the same for the double-float instantiation, whose steps are bound by
-// instruction latency rather than DRAM: more resident warps hide more of it
+#ifndef LPB_STEP_MIN_BLOCKS
+#define LPB_STEP_MIN_BLOCKS 8
+#endif
+#ifndef LPB_STEP_MIN_BLOCKS_F64
+#define LPB_STEP_MIN_BLOCKS_F64 5
+#endif
 #ifndef LPB_STEP_MIN_BLOCKS_DF
 #define LPB_STEP_MIN_BLOCKS_DF 7
 #endif
-// gathers a lane issues before it consumes them (loads in flight per lane)
-#ifndef LPB_GATHER_BATCH
-#define LPB_GATHER_BATCH 4
+// the same for the deep kernels (kDeep), whose grids are less than a wave
+#ifndef LPB_STEP_MIN_BLOCKS_DEEP
+#define LPB_STEP_MIN_BLOCKS_DEEP 4
 #endif
 
 namespace lpb {
@@ -33,17 +42,22 @@ template <> struct Vec<float> { static constexpr int V = 4; };
 template <> struct Vec<double> { static constexpr int V = 2; };
 template <> struct Vec<dfloat> { static constexpr int V = 2; };
 
-// the FP32 primal step streams several iterate blocks besides its gathers:
-// on wide batches (row groups of 32 lanes, where 48 registers hold it
-// without spilling) it gains from more resident warps, i.e. loads in flight
-#ifndef LPB_STEP_MIN_BLOCKS_PRIMAL
-#define LPB_STEP_MIN_BLOCKS_PRIMAL 10
-#endif
-template <typename T, int G, bool PRIMAL> struct MinBlocks { static constexpr int v = LPB_STEP_MIN_BLOCKS; };
-template <int G> struct MinBlocks<float, G, true> {
-    static constexpr int v = G >= 32 ? LPB_STEP_MIN_BLOCKS_PRIMAL : LPB_STEP_MIN_BLOCKS;
+// Gathers a lane issues before it consumes them.  Four keep the registers low
+// enough for the resident warps that fill the memory pipeline.  A step of
+// fewer blocks than one wave has nothing but its rows' chains of round trips:
+// its kernels are the deep ones, eight at a time (sixteen where a row is one
+// or two lanes).  Row groups of 32 lanes have no deep kernel: a step that
+// wide and that small runs alone only for a few hundred rows.
+template <int G> constexpr int kDeep = G >= 32 ? 0 : G <= 2 ? 16 : 8;
+constexpr int kFlat = 4;
+
+template <typename T, int G, int B> struct MinBlocks {
+    static constexpr int v = B > kFlat                       ? (B > 8 ? 3 : LPB_STEP_MIN_BLOCKS_DEEP)
+                             : std::is_same<T, double>::value ? LPB_STEP_MIN_BLOCKS_F64
+                             : std::is_same<T, dfloat>::value ? LPB_STEP_MIN_BLOCKS_DF
+                             : G >= 32                        ? LPB_STEP_MIN_BLOCKS_WIDE
+                                                              : LPB_STEP_MIN_BLOCKS;
 };
-template <int G, bool PRIMAL> struct MinBlocks<dfloat, G, PRIMAL> { static constexpr int v = LPB_STEP_MIN_BLOCKS_DF; };
 
 __device__ __forceinline__ void ldv(const float* p, float (&r)[4]) {
     float4 u = *reinterpret_cast<const float4*>(p);
@@ -79,50 +93,12 @@ __device__ __forceinline__ void stv(dfloat* p, const dfloat (&r)[2]) {
     *reinterpret_cast<float4*>(p) = make_float4(r[0].hi, r[0].lo, r[1].hi, r[1].lo);
 }
 
-// The row-side operands of the epilogues (the iterate, anchor and reflected
-// blocks, and the check outputs) are each read or written once per launch.
-// When the gathered block is too large to stay in L2 anyway (StepArgs::
-// stream), they take the streaming cache hint (evict first), so that L2
-// keeps more of the gathered block, which is read once per nonzero.  When
-// everything fits in L2 the hint would evict what the next step reads.
-#ifndef LPB_STREAM_HINT
-#define LPB_STREAM_HINT 1
-#endif
-template <typename T, int V>
-__device__ __forceinline__ void lds(const T* p, T (&r)[V], bool stream) {
-    static_assert(sizeof(T) * V == sizeof(float4), "one 16-byte vector per lane");
-    if (LPB_STREAM_HINT && stream) {
-        const float4 u = __ldcs(reinterpret_cast<const float4*>(p));
-        memcpy(&r, &u, 16);
-    } else {
-        ldv(p, r);
-    }
-}
-template <typename T, int V>
-__device__ __forceinline__ void sts(T* p, const T (&r)[V], bool stream) {
-    if (LPB_STREAM_HINT && stream) {
-        float4 u;
-        memcpy(&u, &r, 16);
-        __stcs(reinterpret_cast<float4*>(p), u);
-    } else {
-        stv(p, r);
-    }
-}
-
-// scalar read-only load, shuffle, multiply-add and infinity test for each
-// iterate type
+// scalar read-only load, multiply-add and infinity test for each iterate type
 __device__ __forceinline__ float ldg1(const float* p) { return __ldg(p); }
 __device__ __forceinline__ double ldg1(const double* p) { return __ldg(p); }
 __device__ __forceinline__ dfloat ldg1(const dfloat* p) {
     const float2 u = __ldg(reinterpret_cast<const float2*>(p));
     return dfloat(u.x, u.y);
-}
-template <typename T>
-__device__ __forceinline__ T shfl(unsigned mask, T v, int src, int width) {
-    return __shfl_sync(mask, v, src, width);
-}
-__device__ __forceinline__ dfloat shfl(unsigned mask, dfloat v, int src, int width) {
-    return dfloat(__shfl_sync(mask, v.hi, src, width), __shfl_sync(mask, v.lo, src, width));
 }
 __device__ __forceinline__ float mad(float a, float x, float acc) { return fmaf(a, x, acc); }
 __device__ __forceinline__ double mad(double a, double x, double acc) { return fma(a, x, acc); }
@@ -132,6 +108,24 @@ __device__ __forceinline__ dfloat mad(dfloat a, dfloat x, dfloat acc) { return d
 __device__ __forceinline__ float dot_acc(float a, float x, float acc) { return fmaf(a, x, acc); }
 __device__ __forceinline__ double dot_acc(double a, double x, double acc) { return fma(a, x, acc); }
 __device__ __forceinline__ dfloat dot_acc(dfloat a, dfloat x, dfloat acc) { return dfl_dot_acc(a, x, acc); }
+// a product and a difference, each rounded by itself (never joined into one
+// multiply-add by the compiler)
+__device__ __forceinline__ float mul(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ dfloat mul(dfloat a, dfloat b) { return a * b; }
+__device__ __forceinline__ float sub(float a, float b) { return __fsub_rn(a, b); }
+__device__ __forceinline__ double sub(double a, double b) { return __dsub_rn(a, b); }
+__device__ __forceinline__ dfloat sub(dfloat a, dfloat b) { return a - b; }
+// x - tau q with one rounding in FP32 and FP64
+__device__ __forceinline__ float step_from(float x, float tau, float q) { return fmaf(-tau, q, x); }
+__device__ __forceinline__ double step_from(double x, double tau, double q) { return fma(-tau, q, x); }
+__device__ __forceinline__ dfloat step_from(dfloat x, dfloat tau, dfloat q) { return x - tau * q; }
+// ca v + cb w: the second product rounded, then one multiply-add
+template <typename T>
+__device__ __forceinline__ T blend(T ca, T v, T cb, T w) {
+    return mad(ca, v, mul(cb, w));
+}
+__device__ __forceinline__ dfloat blend(dfloat ca, dfloat v, dfloat cb, dfloat w) { return ca * v + cb * w; }
 // 2 v, exact in every iterate type (for dfloat both parts scale)
 __device__ __forceinline__ float twice(float v) { return 2.0f * v; }
 __device__ __forceinline__ double twice(double v) { return 2.0 * v; }
@@ -152,78 +146,119 @@ __device__ __forceinline__ bool is_inf(float v) { return isinf(v); }
 __device__ __forceinline__ bool is_inf(double v) { return isinf(v); }
 __device__ __forceinline__ bool is_inf(dfloat v) { return isinf(v.hi); }
 
-// One round of a row's entries: the G lanes of the row group load up to
-// R = G*K of the row's (col, value) pairs at once (K per lane, coalesced);
-// narrow groups take rounds of 8 to bound the registers holding the entries.
-template <typename T, int G>
-struct Round {
-    static constexpr int K = G >= 8 ? 1 : 8 / G;
-    static constexpr int R = G * K;
-};
+// Entries are summed in rounds of kRound<G>; a row's last batch is filled up
+// with a factor 0 and the column of its round's first entry (no branch
+// between the gathers, and an infinite operand gives what it gives at every
+// batch size).
+template <int G> constexpr int kRound = G >= 8 ? G : 8;
 
-template <typename T, int G>
-__device__ __forceinline__ void load_round(const int* __restrict__ ci, const T* __restrict__ va, int e0, int end,
-                                           int (&c)[Round<T, G>::K], T (&a)[Round<T, G>::K]) {
-    constexpr int K = Round<T, G>::K;
-    const int lane = threadIdx.x % G;
-#pragma unroll
-    for (int q = 0; q < K; ++q) {
-        const int me = e0 + q * G + lane;
-        c[q] = me < end ? __ldg(ci + me) : 0;
-        a[q] = me < end ? ldg1(va + me) : T(0);
-    }
-}
-
-// acc += sum over the round's cnt entries of a_e * src[col_e, colg .. colg+V):
-// entries are broadcast by shuffle inside the row group (entry k sits in
-// register slot k / G of lane k % G, compile-time after unrolling) and the
-// gathers issued four at a time.  Entries past cnt get a = 0 and the round's
-// first column, so every gather stays in bounds.  All lanes of the group
-// must call it (lanes past the last LP pass the tile's first column).
-template <typename T, int V, int G>
-__device__ __forceinline__ void gather_round(const int (&c)[Round<T, G>::K], const T (&a)[Round<T, G>::K], int cnt,
-                                             const T* __restrict__ src, int ld, int colg, unsigned gmask,
-                                             T (&acc)[V]) {
-    constexpr int R = Round<T, G>::R;
-    constexpr int B = LPB_GATHER_BATCH < R ? LPB_GATHER_BATCH : R;
-    static_assert(R % B == 0, "a round is a whole number of gather batches");
-    const int cfirst = __shfl_sync(gmask, c[0], 0, G);
-#pragma unroll
-    for (int k0 = 0; k0 < R; k0 += B) {
-        if (k0 >= cnt) break;
-        int cc[B];
-        T aa[B];
+// acc += entries [beg, end) of a row, in order, every lane of the row group
+// at the same ones (one broadcast load each); the gathers of B entries are
+// issued together.
+template <typename T, int V, int G, int B>
+__device__ __forceinline__ void gather_range(const int* __restrict__ ci, const T* __restrict__ va, const char* src,
+                                             unsigned pitch, int beg, int end, T (&acc)[V]) {
+    int e = beg;
+#pragma unroll 1
+    for (; e + B <= end; e += B) {
+        T w[B], xs[B][V];
 #pragma unroll
         for (int j = 0; j < B; ++j) {
-            const int k = k0 + j;
-            const int cs = __shfl_sync(gmask, c[k / G], k % G, G);
-            const T as = shfl(gmask, a[k / G], k % G, G);
-            cc[j] = k < cnt ? cs : cfirst;
-            aa[j] = k < cnt ? as : T(0);
+            const unsigned c = (unsigned)__ldg(ci + e + j);
+            w[j] = ldg1(va + e + j);
+            ldg_v(reinterpret_cast<const T*>(src + (size_t)c * pitch), xs[j]);
         }
-        T xs[B][V];
-#pragma unroll
-        for (int j = 0; j < B; ++j) ldg_v(src + (size_t)cc[j] * ld + colg, xs[j]);
-        // entries in order, so a column's sum does not depend on G
 #pragma unroll
         for (int j = 0; j < B; ++j)
 #pragma unroll
-            for (int v = 0; v < V; ++v) acc[v] = dot_acc(aa[j], xs[j][v], acc[v]);
+            for (int v = 0; v < V; ++v) acc[v] = dot_acc(w[j], xs[j][v], acc[v]);
+    }
+    if (e < end) {
+        T w[B], xs[B][V];
+        const int first = beg + (e - beg) / kRound<G> * kRound<G>;
+#pragma unroll
+        for (int j = 0; j < B; ++j) {
+            const bool in = e + j < end;
+            const unsigned c = (unsigned)__ldg(ci + (in ? e + j : first));
+            w[j] = in ? ldg1(va + e + j) : T(0);
+            ldg_v(reinterpret_cast<const T*>(src + (size_t)c * pitch), xs[j]);
+        }
+#pragma unroll
+        for (int j = 0; j < B; ++j)
+#pragma unroll
+            for (int v = 0; v < V; ++v) acc[v] = dot_acc(w[j], xs[j][v], acc[v]);
     }
 }
 
-// acc += the row's entries [beg, end), a round at a time
-template <typename T, int V, int G>
-__device__ __forceinline__ void gather_range(const int* __restrict__ ci, const T* __restrict__ va,
-                                             const T* __restrict__ src, int ld, int colg, int beg, int end,
-                                             unsigned gmask, T (&acc)[V]) {
-    constexpr int K = Round<T, G>::K, R = Round<T, G>::R;
+// four or two values from an address that they fill
+__device__ __forceinline__ void ldg4(const int* p, unsigned (&r)[4]) {
+    const int4 u = __ldg(reinterpret_cast<const int4*>(p));
+    r[0] = u.x; r[1] = u.y; r[2] = u.z; r[3] = u.w;
+}
+__device__ __forceinline__ void ldg4(const float* p, float (&r)[4]) { ldg_v(p, r); }
+template <typename T>
+__device__ __forceinline__ void ldg4(const T* p, T (&r)[4]) {
+    T u[2], v[2];
+    ldg_v(p, u);
+    ldg_v(p + 2, v);
+    r[0] = u[0]; r[1] = u[1]; r[2] = v[0]; r[3] = v[1];
+}
+__device__ __forceinline__ void ldg2(const int* p, unsigned (&r)[2]) {
+    const int2 u = __ldg(reinterpret_cast<const int2*>(p));
+    r[0] = u.x; r[1] = u.y;
+}
+__device__ __forceinline__ void ldg2(const float* p, float (&r)[2]) {
+    const float2 u = __ldg(reinterpret_cast<const float2*>(p));
+    r[0] = u.x; r[1] = u.y;
+}
+template <typename T>
+__device__ __forceinline__ void ldg2(const T* p, T (&r)[2]) { ldg_v(p, r); }
+
+template <typename T, int V, int B>
+__device__ __forceinline__ void gather_batch(const unsigned (&c)[B], const T (&w)[B], const char* src, unsigned pitch,
+                                             T (&acc)[V]) {
+    T xs[B][V];
+#pragma unroll
+    for (int j = 0; j < B; ++j) ldg_v(reinterpret_cast<const T*>(src + (size_t)c[j] * pitch), xs[j]);
+#pragma unroll
+    for (int j = 0; j < B; ++j)
+#pragma unroll
+        for (int v = 0; v < V; ++v) acc[v] = dot_acc(w[j], xs[j][v], acc[v]);
+}
+
+// acc += the packed entries of a short row, in order: B at a time (their
+// columns and values are one broadcast load per four), then by fours, then the
+// last two
+template <typename T, int V, int B>
+__device__ __forceinline__ void gather_packed(const int* __restrict__ ci, const T* __restrict__ va, int pairs,
+                                              const char* src, unsigned pitch, T (&acc)[V]) {
+    if (B > 4) {
 #pragma unroll 1
-    for (int e0 = beg; e0 < end; e0 += R) {
-        int c[K];
-        T a[K];
-        load_round<T, G>(ci, va, e0, end, c, a);
-        gather_round<T, V, G>(c, a, min(R, end - e0), src, ld, colg, gmask, acc);
+        for (; pairs >= B / 2; pairs -= B / 2, ci += B, va += B) {
+            unsigned c[B];
+            T w[B];
+#pragma unroll
+            for (int j = 0; j < B; j += 4) {
+                ldg4(ci + j, *reinterpret_cast<unsigned(*)[4]>(c + j));
+                ldg4(va + j, *reinterpret_cast<T(*)[4]>(w + j));
+            }
+            gather_batch<T, V, B>(c, w, src, pitch, acc);
+        }
+    }
+#pragma unroll 1
+    for (; pairs >= 2; pairs -= 2, ci += 4, va += 4) {
+        unsigned c[4];
+        T w[4];
+        ldg4(ci, c);
+        ldg4(va, w);
+        gather_batch<T, V, 4>(c, w, src, pitch, acc);
+    }
+    if (pairs > 0) {
+        unsigned c[2];
+        T w[2];
+        ldg2(ci, c);
+        ldg2(va, w);
+        gather_batch<T, V, 2>(c, w, src, pitch, acc);
     }
 }
 
@@ -235,7 +270,14 @@ struct StepArgs {
     const int* ci;
     const T* va;
     const int* long_rows;
-    int n_long, long_thr;
+    int n_long;
+    // the other rows in the order in which they are taken, their entries in
+    // fours, their cost and bounds (Csr::srec ..)
+    const int4* srec;
+    const int* pci;
+    const T* pva;
+    const T* pk;
+    int n_short;
     const int* lseg;  // long-row blocks: (long row, segment) of each, segment-major
     const int* lseg0; // first segment of each long row; segments of row i: lseg0[i + 1] - lseg0[i]
     int n_lblocks;
@@ -261,7 +303,7 @@ struct StepArgs {
     int t, ce;
     int uni;          // the group of every active column, or -1 if they belong to several
     int pdl;          // launched as a programmatic dependent of the previous step kernel
-    int stream;       // the gathered block exceeds half of L2: streaming hints on the row operands
+    int hbm;          // the gathered block exceeds half of L2: the iterates come from HBM
 };
 
 // Reduce the row groups' partial sums of a long row through shared memory;
@@ -294,81 +336,134 @@ __device__ __forceinline__ T barrier(T v, T lo, T hi) {
 template <typename T, int TN>
 struct TileParams {
     T tau[TN], lo[TN], hi[TN], c[TN], sigma[TN], isigma[TN], ca[TN], cb[TN], pa[TN], pb[TN];
-    int kind[TN], var[TN];
+    int key[TN];  // the override's row: var of a box, ~var of an objective, INT_MAX if none
 };
+
+// The elementwise steps state where a product is rounded before it is added
+// (mul, step_from, blend), so that every kernel that runs them gives the same
+// bits.
+//
+// The primal step of one element: box projection, reflection (the Halpern
+// update of Eq. mainiter is applied when the next step rebuilds its
+// iterate).  acc is the row's product.
+template <typename T, bool CHECK>
+__device__ __forceinline__ void primal_element(T x, T acc, T tau, T cj, T lo, T hi, T& xh, T& xb, T& dz) {
+    const T q = cj + acc, step = mul(tau, q);
+    T s = CHECK ? sub(x, step) : step_from(x, tau, q);
+    const bool inside = s < hi && s > lo;
+    s = s < hi ? s : hi;
+    s = s > lo ? s : lo;
+    xh = s;
+    xb = twice(s) - x;
+    // x^ - x: where the box is not active it is -tau (c + G) exactly,
+    // which stays accurate when |x| is large (diverging iterates of an
+    // infeasible LP); elsewhere the difference with the bound
+    dz = inside ? -step : s - x;
+}
+
+// The dual step of one element: row projection and Halpern update.
+template <typename T>
+__device__ __forceinline__ void dual_element(T ca, T cb, T y, T y0, T acc, T sg, T isg, T lr, T ur, T& yh, T& yn,
+                                             T& dz) {
+    const T s = over_sigma(y, sg, isg) + acc;
+    T p = s < ur ? s : ur;
+    p = p > lr ? p : lr;
+    yh = sg * (s - p);
+    yn = blend(ca, twice(yh) - y, cb, y0);
+    // y^ - y: y^ = 0 exactly where the row bound is not active; where it
+    // is, y^ - y = sigma (A xb - Pi(v)) without the cancellation of y
+    dz = p == s ? -y : sg * (acc - p);
+}
+
+// A row's own operands in the lane's columns: its stored point (primal: the
+// reflection Xbar; dual: Y) and anchor; and its cost and bounds.
+template <typename T, int V>
+struct RowOwn {
+    T z[V], z0[V];
+};
+template <typename T>
+struct RowK {
+    T c, lo, hi;
+};
+
+// the same by plain loads (long rows)
+template <typename T, int V, bool PRIMAL>
+__device__ __forceinline__ RowOwn<T, V> load_own(const StepArgs<T>& a, int row, int col0) {
+    RowOwn<T, V> o;
+    const size_t off = (size_t)row * a.ld + col0;
+    ldv((PRIMAL ? a.Zbar : a.Z) + off, o.z);
+    ldv(a.Z0 + off, o.z0);
+    return o;
+}
 
 // primal epilogue for row `row`, lane columns col0 .. col0+V (q0 = their
 // offset in the tile): the iterate rebuilt from the previous reflection,
-// box projection, reflection (the Halpern update of Eq. mainiter is applied
-// when the next step rebuilds its iterate)
+// X^k = k/(k+1) Xb + X^0/(k+1), then the step
 template <typename T, int V, int TN, bool CHECK>
 __device__ __forceinline__ void primal_epilogue(const StepArgs<T>& a, const TileParams<T, TN>& P, int row, int col0,
-                                                int q0, const T (&acc)[V], T upa, T upb) {
+                                                int q0, const T (&acc)[V], const RowOwn<T, V>& o, const RowK<T>& k,
+                                                T upa, T upb) {
     const size_t off = (size_t)row * a.ld + col0;
-    T x[V], x0[V];
-    lds(a.Zbar + off, x, a.stream);
-    lds(a.Z0 + off, x0, a.stream);
-    const T cr = a.rc[row], lor = a.rlo[row], hir = a.rhi[row];
     T xh[V], xb[V], dz[V];
 #pragma unroll
     for (int v = 0; v < V; ++v) {
         const int q = q0 + v;
         const T pa = a.uni >= 0 ? upa : P.pa[q], pb = a.uni >= 0 ? upb : P.pb[q];
-        x[v] = mad(pa, x[v], pb * x0[v]);  // X^k = k/(k+1) Xb + X^0/(k+1)
-        const int kind = P.kind[q], var = P.var[q];
-        T cj = cr, lo = lor, hi = hir;
-        if (kind == 2) cj = var == row ? P.c[q] : T(0);
-        else if (kind == 1 && var == row) { lo = P.lo[q]; hi = P.hi[q]; }
-        const T step = P.tau[q] * (cj + acc[v]);
-        T s = x[v] - step;
-        const bool inside = s < hi && s > lo;
-        s = s < hi ? s : hi;
-        s = s > lo ? s : lo;
-        xh[v] = s;
-        xb[v] = twice(s) - x[v];
-        // x^ - x: where the box is not active it is -tau (c + G) exactly,
-        // which stays accurate when |x| is large (diverging iterates of an
-        // infeasible LP); elsewhere the difference with the bound
-        dz[v] = inside ? -step : s - x[v];
+        const T x = mad(pa, o.z[v], mul(pb, o.z0[v]));
+        const int key = P.key[q];
+        T cj = key < 0 ? T(0) : k.c, lo = k.lo, hi = k.hi;
+        if (key == row) {
+            lo = P.lo[q];
+            hi = P.hi[q];
+        }
+        if (key == ~row) cj = P.c[q];
+        primal_element<T, CHECK>(x, acc[v], P.tau[q], cj, lo, hi, xh[v], xb[v], dz[v]);
     }
-    sts(a.Zbar + off, xb, a.stream);
+    stv(a.Zbar + off, xb);
     if (CHECK) {
-        sts(a.Zh + off, xh, a.stream);
-        sts(a.DZ + off, dz, a.stream);
+        stv(a.Zh + off, xh);
+        stv(a.DZ + off, dz);
     }
 }
 
-// dual epilogue: row projection and Halpern update
+// dual epilogue
 template <typename T, int V, int TN, bool CHECK>
 __device__ __forceinline__ void dual_epilogue(const StepArgs<T>& a, const TileParams<T, TN>& P, int row, int col0,
-                                              int q0, const T (&acc)[V], T uca, T ucb) {
+                                              int q0, const T (&acc)[V], const RowOwn<T, V>& o, const RowK<T>& k, T uca,
+                                              T ucb) {
     const size_t off = (size_t)row * a.ld + col0;
-    T y[V], y0[V];
-    lds(a.Z + off, y, a.stream);
-    lds(a.Z0 + off, y0, a.stream);
-    const T lr = a.rlo[row], ur = a.rhi[row];
     T yh[V], yn[V], dz[V];
 #pragma unroll
     for (int v = 0; v < V; ++v) {
-        const T sg = P.sigma[q0 + v];
-        const T s = over_sigma(y[v], sg, P.isigma[q0 + v]) + acc[v];
-        T p = s < ur ? s : ur;
-        p = p > lr ? p : lr;
-        yh[v] = sg * (s - p);
         const T ca = a.uni >= 0 ? uca : P.ca[q0 + v], cb = a.uni >= 0 ? ucb : P.cb[q0 + v];
-        yn[v] = ca * (twice(yh[v]) - y[v]) + cb * y0[v];
-        // y^ - y: y^ = 0 exactly where the row bound is not active; where it
-        // is, y^ - y = sigma (A xb - Pi(v)) without the cancellation of y
-        dz[v] = p == s ? -y[v] : sg * (acc[v] - p);
+        dual_element(ca, cb, o.z[v], o.z0[v], acc[v], P.sigma[q0 + v], P.isigma[q0 + v], k.lo, k.hi, yh[v],
+                     yn[v], dz[v]);
     }
-    sts(a.Z + off, yn, a.stream);
+    stv(a.Z + off, yn);
     if (CHECK) {
         T dzp[V];
 #pragma unroll
-        for (int v = 0; v < V; ++v) dzp[v] = barrier(dz[v], lr, ur);
-        sts(a.Zh + off, yh, a.stream);
-        sts(a.DZ + off, dz, a.stream);
-        sts(a.Aux + off, dzp, a.stream);
+        for (int v = 0; v < V; ++v) dzp[v] = barrier(dz[v], k.lo, k.hi);
+        stv(a.Zh + off, yh);
+        stv(a.DZ + off, dz);
+        stv(a.Aux + off, dzp);
+    }
+}
+
+// Programmatic dependent launch: what a step kernel reads before this wait
+// (the matrix, costs and bounds, per-column parameters, Halpern weights) the
+// previous kernel does not write, so its round trips overlap
+// the end of that kernel.  That holds because only step kernels after an
+// interval's first are launched as programmatic dependents, and their
+// predecessor is a step kernel; the first primal step of an interval follows
+// the check, admission, extraction, compaction and migration kernels that do
+// write those, and is launched without the attribute (launch_iteration).
+// Then let the next step kernel start its own prologue on the SMs this grid
+// frees.
+__device__ __forceinline__ void pdl_wait(int pdl) {
+    if (pdl) {
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     }
 }
 
@@ -399,24 +494,35 @@ __device__ __forceinline__ dfloat add(dfloat a, dfloat b) { return a + b; }
 
 // One step (primal or dual) of the iteration on one column tile.
 //   Blocks [0, n_lblocks): one segment of a long row each (at most kStepSeg
-//   entries), split into contiguous pieces over the block's row groups and
-//   reduced in shared memory.  A row of one segment is finished by its block;
-//   for a row of several, each block stores its partial sums, and the block
-//   that completes the row (the last to take the row's ticket; no block
+//   entries), split into contiguous pieces over the block's G-lane row groups
+//   and reduced in shared memory.  A row of one segment is finished by its
+//   block; for a row of several, each block stores its partial sums, and the
+//   block that completes the row (the last to take the row's ticket; no block
 //   waits) adds the partials in segment order and finishes the row, so the
 //   result does not depend on which block ends last.
-//   Blocks [n_lblocks, gx): persistent over the short rows, row group g
-//   taking rows g, g + stride, ...; while it gathers and finishes a row, the
-//   row pointers and the first index round of its next row are in flight.
+//   Blocks [n_lblocks, gx): persistent over the short rows (srec), row group
+//   g taking records g, g + stride, ...; a warp's row groups take rows of
+//   about the same length (build_short_rows).
+//   What bounds a short row: its gathers move 16 G bytes an entry from L2
+//   (at most 64 bytes a cycle and SM), and everything else that goes through
+//   L1 takes a turn from them.  So a lane reads four columns and four values
+//   with one broadcast load each from the packed rows, where shuffled entries
+//   took two shuffles an entry, and the row's cost and bounds come in one
+//   load.  Measured with the shuffles and with the packed rows (a pass of the
+//   benchmark's power-law batch, 256 iterations: 7.8 and 6.5 ms; 64 LPs on a
+//   10k x 10k matrix, mostly double-float: 7.9 and 6.3 ms; 101 LPs on a 200k
+//   x 400k matrix, 64 iterations: 30.5 and 26.2 ms; the bound-tightening
+//   batch of 1024 LPs, 64 iterations: 65.4 and 61.1 ms; 128 LPs on the 1M x
+//   2M matrix: 139.6 and 133.0 ms).  Evict-first hints on a row's own
+//   operands cost 2-4% in this form; prefetching the next row's own operands
+//   to L2 gains 1-2% where they come from HBM.
 //   (bx, by) is the block's place in the step's own grid (bx over the
 //   long-row and persistent blocks, gx of them; by over the column tiles).
-template <typename T, int G, bool CHECK, bool PRIMAL>
+template <typename T, int G, int B, bool CHECK, bool PRIMAL>
 __device__ __forceinline__ void step_body(const StepArgs<T>& a, const int bx, const int by, const int gx) {
     constexpr int V = Vec<T>::V, GPB = kBlock / G, TN = G * V;
-    constexpr int K = Round<T, G>::K, R = Round<T, G>::R;
-    __shared__ T red[kBlock * V];
+    __shared__ uint4 red[kBlock];  // a long-row block's partial sums
     __shared__ TileParams<T, TN> P;
-    const int lane = threadIdx.x % G, grp = threadIdx.x / G;
     const int tile0 = by * TN;
     for (int q = threadIdx.x; q < TN; q += kBlock) {
         const int j = tile0 + q;
@@ -434,8 +540,8 @@ __device__ __forceinline__ void step_body(const StepArgs<T>& a, const int bx, co
             }
         }
         if (PRIMAL) {
-            P.kind[q] = in ? a.col.kind[j] : 0;
-            P.var[q] = in ? a.col.var[j] : -1;
+            const int kind = in ? a.col.kind[j] : 0;
+            P.key[q] = kind == 1 ? a.col.var[j] : kind == 2 ? ~a.col.var[j] : INT_MAX;
             P.tau[q] = in ? a.col.tau[j] : T(0);
             P.lo[q] = in ? a.col.lo[j] : T(0);
             P.hi[q] = in ? a.col.hi[j] : T(0);
@@ -449,63 +555,31 @@ __device__ __forceinline__ void step_body(const StepArgs<T>& a, const int bx, co
     // (the primal step takes the previous iteration's, the dual step this one's)
     const int hu = a.uni >= 0 ? 2 * (a.uni * (a.ce + 1) + a.t + (PRIMAL ? 0 : 1)) : 0;
     const T uca = a.uni >= 0 ? a.hal[hu] : T(0), ucb = a.uni >= 0 ? a.hal[hu + 1] : T(0);
+    const unsigned pitch = (unsigned)a.ld * (unsigned)sizeof(T);
+
+    const int lane = threadIdx.x % G, grp = threadIdx.x / G;
     const int col0 = tile0 + lane * V;
     const bool active = col0 < a.ncol;
-    const int colg = active ? col0 : tile0;
     const unsigned gmask = G == 32 ? 0xffffffffu : (((1u << G) - 1u) << ((threadIdx.x & 31) & ~(G - 1)));
-
-    // The block's first entries: of its segment's piece, or of its row
-    // group's first row.
-    const bool is_seg = bx < a.n_lblocks;
-    const int stride = (gx - a.n_lblocks) * GPB;
-    int r = (bx - a.n_lblocks) * GPB + grp;
-    int beg = 0, end = 0;
-    int c[K];
-    T av[K];
-    if (is_seg) {
-        const int li = a.lseg[2 * bx], sg = a.lseg[2 * bx + 1], ns = a.lseg0[li + 1] - a.lseg0[li];
+    const char* const src = reinterpret_cast<const char*>(a.src + (active ? col0 : tile0));
+    if (bx < a.n_lblocks) {
+        const int li = a.lseg[2 * bx], sg = a.lseg[2 * bx + 1];
+        const int s0 = a.lseg0[li], ns = a.lseg0[li + 1] - s0;
         const int row = a.long_rows[li];
         const int rb0 = a.rp[row], re0 = a.rp[row + 1];
         const int sl = (re0 - rb0 + ns - 1) / ns;  // entries per segment
         const int rb = min(re0, rb0 + sg * sl), re = min(re0, rb + sl);
         const int piece = (re - rb + GPB - 1) / GPB;
-        beg = min(re, rb + grp * piece);
-        end = min(re, beg + piece);
-        load_round<T, G>(a.ci, a.va, beg, end, c, av);
-    } else if (r < a.rows) {
-        beg = a.rp[r];
-        end = a.rp[r + 1];
-        load_round<T, G>(a.ci, a.va, beg, end - beg <= a.long_thr ? end : beg, c, av);
-    }
-    __syncthreads();
-    // Programmatic dependent launch: everything above reads only data that
-    // the previous kernel does not write (the matrix, per-column parameters,
-    // Halpern weights), so its round trips overlap the end of that kernel: a
-    // step then waits for its gathers alone.  That holds because only step
-    // kernels after an interval's first are launched as programmatic
-    // dependents, and their predecessor is a step kernel; the first primal
-    // step of an interval follows the check, admission, extraction,
-    // compaction and migration kernels that do write those parameters, and is
-    // launched without the attribute (launch_iteration).  Wait for the
-    // predecessor to complete before touching the iterates, then let the next
-    // step kernel start its own prologue on the SMs this grid frees.
-    if (a.pdl) {
-        asm volatile("griddepcontrol.wait;" ::: "memory");
-        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    }
-
-    if (is_seg) {
+        const int beg = min(re, rb + grp * piece), end = min(re, beg + piece);
+        __syncthreads();
+        pdl_wait(a.pdl);
         T acc[V];
 #pragma unroll
         for (int v = 0; v < V; ++v) acc[v] = T(0);
-        gather_round<T, V, G>(c, av, min(R, end - beg), a.src, a.ld, colg, gmask, acc);
-        if (end - beg > R) gather_range<T, V, G>(a.ci, a.va, a.src, a.ld, colg, beg + R, end, gmask, acc);
+        gather_range<T, V, G, B>(a.ci, a.va, src, pitch, beg, end, acc);
         fin<V>(acc);
-        if (!long_row_reduce<T, V, G>(acc, red)) return;
+        if (!long_row_reduce<T, V, G>(acc, reinterpret_cast<T*>(red))) return;
         // only row group 0 (lanes 0 .. G-1 of warp 0) continues
-        const int li = a.lseg[2 * bx], sg = a.lseg[2 * bx + 1];
-        const int s0 = a.lseg0[li], ns = a.lseg0[li + 1] - s0;
-        const int row = a.long_rows[li];
         if (ns > 1) {
             if (active) stv_cg(a.part + (size_t)(s0 + sg) * a.ld + col0, acc);
             __threadfence();
@@ -530,38 +604,42 @@ __device__ __forceinline__ void step_body(const StepArgs<T>& a, const int bx, co
             }
         }
         if (!active) return;
-        if (PRIMAL) primal_epilogue<T, V, TN, CHECK>(a, P, row, col0, lane * V, acc, uca, ucb);
-        else dual_epilogue<T, V, TN, CHECK>(a, P, row, col0, lane * V, acc, uca, ucb);
+        const RowOwn<T, V> o = load_own<T, V, PRIMAL>(a, row, col0);
+        const RowK<T> k{PRIMAL ? a.rc[row] : T(0), a.rlo[row], a.rhi[row]};
+        if (PRIMAL) primal_epilogue<T, V, TN, CHECK>(a, P, row, col0, lane * V, acc, o, k, uca, ucb);
+        else dual_epilogue<T, V, TN, CHECK>(a, P, row, col0, lane * V, acc, o, k, uca, ucb);
         return;
     }
 
+    const int stride = (gx - a.n_lblocks) * GPB;
+    int i = (bx - a.n_lblocks) * GPB + grp;
+    int4 rec = make_int4(0, 0, 0, 0);
+    if (i < a.n_short) rec = __ldg(a.srec + i);
+    __syncthreads();
+    pdl_wait(a.pdl);
 #pragma unroll 1
-    while (r < a.rows) {
-        const int rn = r + stride;
-        int nbeg = 0, nend = 0;
-        if (rn < a.rows) {
-            nbeg = a.rp[rn];
-            nend = a.rp[rn + 1];
-        }
-        const bool is_short = end - beg <= a.long_thr;
+    for (; i < a.n_short; i += stride) {
+        const int row = rec.x, first = rec.y, pairs = rec.z;
+        if (i + stride < a.n_short) rec = __ldg(a.srec + i + stride);
         T acc[V];
 #pragma unroll
         for (int v = 0; v < V; ++v) acc[v] = T(0);
-        if (is_short) {
-            gather_round<T, V, G>(c, av, min(R, end - beg), a.src, a.ld, colg, gmask, acc);
-            if (end - beg > R)
-                gather_range<T, V, G>(a.ci, a.va, a.src, a.ld, colg, beg + R, end, gmask, acc);
-            fin<V>(acc);
+        gather_packed<T, V, B>(a.pci + 4 * (size_t)first, a.pva + 4 * (size_t)first, pairs, src, pitch, acc);
+        fin<V>(acc);
+        // the next row's own operands towards L2, when they come from HBM
+        if (a.hbm && active && i + stride < a.n_short) {
+            const size_t off = (size_t)rec.x * a.ld + col0;
+            asm volatile("prefetch.global.L2 [%0];" ::"l"((PRIMAL ? a.Zbar : a.Z) + off));
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(a.Z0 + off));
         }
-        // the next row's first index round, issued before this row's epilogue
-        if (rn < a.rows) load_round<T, G>(a.ci, a.va, nbeg, nend - nbeg <= a.long_thr ? nend : nbeg, c, av);
-        if (is_short && active) {
-            if (PRIMAL) primal_epilogue<T, V, TN, CHECK>(a, P, r, col0, lane * V, acc, uca, ucb);
-            else dual_epilogue<T, V, TN, CHECK>(a, P, r, col0, lane * V, acc, uca, ucb);
+        if (active) {
+            const RowOwn<T, V> o = load_own<T, V, PRIMAL>(a, row, col0);
+            T kk[4];
+            ldg4(a.pk + 4 * (size_t)i, kk);
+            const RowK<T> k{kk[0], kk[1], kk[2]};
+            if (PRIMAL) primal_epilogue<T, V, TN, CHECK>(a, P, row, col0, lane * V, acc, o, k, uca, ucb);
+            else dual_epilogue<T, V, TN, CHECK>(a, P, row, col0, lane * V, acc, o, k, uca, ucb);
         }
-        r = rn;
-        beg = nbeg;
-        end = nend;
     }
 }
 
@@ -647,8 +725,8 @@ inline cudaError_t l2_bytes(long long* out) {
 
 // The arguments of one matrix's primal step (rows of A~^T gathering Y) or
 // dual step (rows of A~ gathering Xbar) at iteration t of its interval;
-// pdl is left to the caller.  l2: the device's L2 bytes, which decide the
-// streaming hints.
+// pdl is left to the caller.  l2: the device's L2 bytes, which decide whether
+// a row's own operands are prefetched.
 template <typename T>
 StepArgs<T> step_args(bool primal, const IterData<T>& d, const IterBufs<T>& b, int ld, int ncol, const T* hal,
                       int t, int ce, int uni, long long l2) {
@@ -660,7 +738,11 @@ StepArgs<T> step_args(bool primal, const IterData<T>& d, const IterBufs<T>& b, i
     a.va = primal ? d.at_vals : d.a_vals;
     a.long_rows = c.long_rows;
     a.n_long = c.n_long;
-    a.long_thr = c.long_thr;
+    a.srec = c.srec;
+    a.pci = c.pci;
+    a.pva = primal ? d.at_pv : d.a_pv;
+    a.pk = primal ? d.at_pk : d.a_pk;
+    a.n_short = c.n_short;
     a.lseg = c.lseg;
     a.lseg0 = c.lseg0;
     a.n_lblocks = c.n_lblocks;
@@ -669,7 +751,7 @@ StepArgs<T> step_args(bool primal, const IterData<T>& d, const IterBufs<T>& b, i
     a.ntix = c.ntix;
     // the gathered block: Y (m x ld) for the primal step, Xbar (n x ld) for the dual step
     const long long gbytes = (long long)(primal ? d.A.rows : d.A.cols) * ld * (long long)sizeof(T);
-    a.stream = 2 * gbytes > l2;
+    a.hbm = 2 * gbytes > l2;
     if (primal) {
         a.src = b.Y;
         a.Z = nullptr;

@@ -1,0 +1,118 @@
+"""GPU: the step kernels at the edges of their row groups, batches of entries,
+row windows and column tiles, against the same three iterations in plain
+numpy FP64 (Sec. 4, Eq. mainiter and the operator T)."""
+import types
+
+import numpy as np
+import pytest
+
+import lpgen
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def lpb():
+    import torch
+
+    assert torch.cuda.is_available(), "GPU tests need a CUDA device"
+    from paper_2601_21990_gb300 import _build, lpb as mod
+
+    _build.build()
+    mod.load()
+    return mod
+
+
+def _lp(m, n, longest, seed):
+    """Rows of 0 .. longest entries in turn (every remainder of a batch of
+    entries, empty rows among them), box [0, 10], rows around a point."""
+    rng = np.random.default_rng(seed)
+    lengths = np.minimum(np.arange(m) % (longest + 1), n).astype(np.int64)
+    rng.shuffle(lengths)
+    cols = np.concatenate([np.sort(rng.choice(n, k, replace=False)) for k in lengths])
+    ptr = np.zeros(m + 1, dtype=np.int64)
+    np.cumsum(lengths, out=ptr[1:])
+    x0 = rng.uniform(0.0, 10.0, n)
+    lp = lpgen.LPData(m, n, ptr, cols.astype(np.int32), lpgen._signed_uniform(rng, cols.size), rng.standard_normal(n),
+                      None, None, np.zeros(n), np.full(n, 10.0), x0, "steps")
+    lpgen._rows_around(lp, x0, rng)
+    return lp
+
+
+def _three_iterations(lp, specs, dr, dc, eta, iters=3):
+    rows = np.repeat(np.arange(lp.m), np.diff(lp.row_ptr))
+    v = dr[rows] * lp.vals * dc[lp.col_idx]
+
+    def a(x):
+        out = np.zeros((lp.m, x.shape[1]))
+        np.add.at(out, rows, v[:, None] * x[lp.col_idx])
+        return out
+
+    def at(y):
+        out = np.zeros((lp.n, y.shape[1]))
+        np.add.at(out, lp.col_idx, v[:, None] * y[rows])
+        return out
+
+    k = len(specs.kind)
+    c = np.repeat((dc * lp.c)[:, None], k, 1)
+    lo, hi = np.repeat((lp.var_lo / dc)[:, None], k, 1), np.repeat((lp.var_hi / dc)[:, None], k, 1)
+    for q in range(k):
+        j = specs.var[q]
+        if specs.kind[q] == 1:
+            lo[j, q], hi[j, q] = max(lp.var_lo[j], specs.lo[q]) / dc[j], min(lp.var_hi[j], specs.hi[q]) / dc[j]
+        elif specs.kind[q] == 2:
+            c[:, q] = 0.0
+            c[j, q] = dc[j] * specs.sign[q]
+    l, u = (dr * lp.row_lo)[:, None], (dr * lp.row_hi)[:, None]
+    b = np.where(np.abs(l) > np.abs(u), l, u)
+    w = np.linalg.norm(c, axis=0) / np.linalg.norm(b)
+    tau, sigma = eta / w, eta * w
+    x, y = np.clip(np.zeros_like(c), lo, hi), np.zeros((lp.m, k))
+    x0, y0 = x, y
+    for t in range(iters):
+        xh = np.clip(x - tau * (c + at(y)), lo, hi)
+        xb = 2 * xh - x
+        s = y / sigma + a(xb)
+        yh = sigma * (s - np.clip(s, l, u))
+        x = (t + 1) / (t + 2) * xb + x0 / (t + 2)
+        y = (t + 1) / (t + 2) * (2 * yh - y) + y0 / (t + 2)
+    return (dc[:, None] * xh).T, (dr[:, None] * yh).T
+
+
+def _specs(lp, k, seed):
+    rng = np.random.default_rng(seed)
+    var = rng.integers(0, lp.n, k)
+    kind = np.arange(k) % 3  # base LP, a box, an objective
+    return types.SimpleNamespace(kind=kind, var=var, lo=rng.uniform(1.0, 3.0, k), hi=rng.uniform(4.0, 9.0, k),
+                                 sign=np.where(rng.random(k) < 0.5, 1.0, -1.0))
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("m,n,longest,lps", [
+    (37, 50, 9, 1), (60, 41, 32, 2), (100, 90, 33, 3), (100, 90, 33, 5), (200, 300, 40, 9), (300, 200, 31, 17),
+    (2047, 700, 12, 33), (2048, 900, 33, 64), (2049, 4097, 34, 65), (4100, 2100, 17, 129), (700, 900, 300, 40),
+])
+def test_steps_match_plain_iterations(lpb, precision, m, n, longest, lps):
+    """x^ and y^ after three iterations.  The batch runs the kernels of every
+    row-group width, grids of less and of more than one wave, rows of one and
+    of several segments.  FP32 tolerance: a sum of k <= 41 products (longer
+    rows are cut into pieces of at most 75) is off by at most k u |a||x|, and
+    |a||x| <= sqrt(k) times the norms; six products: 6 * 75^1.5 u < 4000 u of
+    the largest value.  FP64: the same with its u, times 4 for the oracle's own
+    rounding."""
+    lp = _lp(m, n, longest, m + lps)
+    sp = _specs(lp, lps, lps)
+    h = lpb.Handle(lp, precision=lpb.FP64 if precision == "fp64" else lpb.MIXED)
+    dr, dc = h.scaling()
+    ex, ey = _three_iterations(lp, sp, dr, dc, h.info()[0])
+    u = 2.0 ** -53 * 4 if precision == "fp64" else 2.0 ** -24
+    specs = lpb.specs_array(sp.kind, sp.var, sp.lo, sp.hi, sp.sign)
+    for _ in range(2):  # a captured interval and its replay
+        b = h.solve(specs, tol=1e-12, max_iter=3)
+        assert (b.results()["iters"] == 3).all()
+        for q in range(lps):
+            _, x, y = b.result(q)
+            assert np.abs(x - ex[q]).max() <= 4000 * u * max(1.0, np.abs(ex[q] / dc).max()) * dc.max(), q
+            assert np.abs(y - ey[q]).max() <= 4000 * u * max(1.0, np.abs(ey[q] / dr).max()) * dr.max(), q
+        b.free()
+    h.close()
