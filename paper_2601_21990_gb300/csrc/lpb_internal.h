@@ -96,10 +96,6 @@ struct Csr {
     int ntix = 0;
 };
 
-#ifndef LPB_LONG_SEG
-#define LPB_LONG_SEG 1024
-#endif
-constexpr int kLongSeg = LPB_LONG_SEG;  // rows longer than this get a block in the power iteration
 // Entries per segment of a long row in the step kernels.  Segments are
 // listed segment-major, so the blocks resident together gather from a
 // window of columns about (resident blocks / long rows) segments wide: with
@@ -198,8 +194,9 @@ cudaError_t ruiz_pock_chambolle(const Csr& a, const double* a_vals, const Csr& a
                                 double* tmp_r, double* tmp_c, cudaStream_t s);
 cudaError_t scale_values(const Csr& a, const double* a_vals, const double* d_r, const double* d_c,
                          bool rows_are_constraints, double* out64, float* out32, cudaStream_t s);
-// doubles of device work space power_norm needs for an m x n matrix of nnz entries
-size_t power_work_doubles(int m, int n, long long nnz, int max_iter);
+// doubles of device work space power_norm needs for an m x n matrix
+size_t power_work_doubles(int m, int n, int max_iter);
+// (a and at list their rows of more than kLongRow entries)
 cudaError_t power_norm(const Csr& a, const Csr& at, int max_iter, double tol, uint64_t seed,
                        double* work, double* est_out, int* iters_out, cudaStream_t s);
 cudaError_t scale_vectors(int m, int n, const double* d_r, const double* d_c, const double* c,

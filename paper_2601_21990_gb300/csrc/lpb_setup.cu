@@ -450,132 +450,218 @@ __global__ void k_power_init(double* v, int n, uint64_t seed) {
 }
 
 // One product of A~^T A~ takes two launches of k_power_spmv.  Each block
-// leaves its share of the squared norm of the result as one partial; the
-// last block to finish (an atomic ticket, no waiting) adds the partials in
-// block order and writes the norm to a scalar the next launch reads.  The
-// grid is fixed at kPowBlocks plus one block per long row, so the rows each
-// block covers and the order of every sum are the same on every run.  The normalisation v = w / ||w|| is
-// applied after the forward product, u = (A~ w) / ||w||, so no launch writes
-// v and none only reduces.
+// leaves its share of the squared norm of the result as one partial, and the
+// next launch adds the partials in block order: the forward launch in every
+// block (it scales by the norm), the other in its first block (which only
+// records it).  The first block decides whether the iteration has stopped;
+// launches queued past that point return at once.  The grid is fixed, so the
+// rows each block covers and the order of every sum are the same on every
+// run.  The vector is kept near unit norm by a power of two, which rounds
+// nothing: u = 2^-e A~ w with e the exponent of ||w||, and the estimate
+// ||A~ w|| / ||w|| = ||u|| / (2^-e ||w||) is formed once.
 //
-// The short-row blocks of a launch: one per kPowRows rows, at least
-// kPowBlocks and at most kPowBlocksMax (a function of the row count alone,
-// so still the same on every run).  Each row group walks its rows one after
-// another, a chain of dependent loads per row: on the 1M x 2M strong-
-// branching matrix the fixed 512 blocks gave each row group 61 (A~) and
-// 122 (A~^T) rows; matrices of up to 131k rows keep 512 blocks, the best of
-// a sweep on the 20k-row and 100k-row matrices.
-#ifndef LPB_POW_BLOCKS
-#define LPB_POW_BLOCKS 512
-#endif
-#ifndef LPB_POW_BLOCKS_MAX
-#define LPB_POW_BLOCKS_MAX 4096
-#endif
-#ifndef LPB_POW_ROWS
-#define LPB_POW_ROWS 256
-#endif
-#ifndef LPB_POW_GROUP
-#define LPB_POW_GROUP 8
-#endif
-constexpr int kPowBlocks = LPB_POW_BLOCKS;
-constexpr int kPowBlocksMax = LPB_POW_BLOCKS_MAX;
-constexpr int kPowRows = LPB_POW_ROWS;
-constexpr int kPowThreads = 256;
-static_assert(kPowBlocks <= kPowBlocksMax, "power grid bounds");
-inline int pow_blocks(int rows) {
-    const long long b = ((long long)rows + kPowRows - 1) / kPowRows;
-    return (int)(b < kPowBlocks ? kPowBlocks : b > kPowBlocksMax ? kPowBlocksMax : b);
-}
-constexpr int kPowGroup = LPB_POW_GROUP;  // lanes per row
-static_assert(kPowGroup >= 1 && kPowGroup <= 32 && (kPowGroup & (kPowGroup - 1)) == 0, "lanes per row: a power of 2");
+// What bounds a launch on a matrix in L2 is the FP64 pipe (a warp's
+// multiply-add takes it 16 cycles; a division by ||w|| per row took some 200)
+// and the chain of round trips around it.  So a short row has few lanes, only
+// the multiply-adds that some lane of a warp needs are issued, the blocks are
+// few and large (one ticket per block, 512 to 3125 of them, took 28 to 48 us
+// a launch), a row group has its next row's entries on their way while it
+// gathers for this one, and the first row's are loaded ahead of the wait for
+// the previous launch (programmatic dependent launch).
+constexpr int kPowBlocks = 152;
+constexpr int kPowThreads = 1024;
+constexpr int kPowGroup = 4;      // lanes of a short row
+constexpr int kPowLong = 1024;    // rows with more entries take a block, other long rows a warp
 
-// The last of the grid's blocks to call this (after writing part[blockIdx.x])
-// sets *nrm = sqrt(sum of the partials in block order), records it at
-// hist[slot] when hist is given, and rearms the ticket.
-__device__ __forceinline__ void finish_norm(double* part, unsigned* __restrict__ ticket,
-                                            double* __restrict__ nrm, double* __restrict__ hist, int slot,
-                                            double* sh) {
-    __shared__ bool last;
-    if (threadIdx.x == 0) {
-        __threadfence();
-        last = atomicAdd(ticket, 1u) == gridDim.x - 1;
-    }
-    __syncthreads();
-    if (!last) return;
-    __threadfence();
+struct PowArgs {
+    const int* rp;
+    const int* ci;
+    const double* v;
+    int rows;
+    const int* mid;         // rows of more than kLongRow entries
+    int n_mid;
+    const int* longs;       // rows of more than kPowLong entries
+    int n_long;
+    const double* x;
+    double* y;
+    const double* pin;      // partials of the operand's squared norm
+    double* pout;
+    double* xnorm;          // forward: the operand's scaled norm, read by the second launch
+    double* est;            // estimate of each product
+    int it;
+    int* stop;
+    double tol;
+};
+
+// 2^-e with e the exponent of v (1 for a v that has none)
+__device__ __forceinline__ double pow2_below(double v) {
+    const long long e = __double_as_longlong(v) >> 52 & 0x7ff;
+    return e >= 1 && e <= 2045 ? __longlong_as_double((2046 - e) << 52) : 1.0;
+}
+
+// sum of part[0 .. count) in a fixed order; warp 0 calls it, the sum is in
+// all its lanes
+__device__ __forceinline__ double warp_sum(const double* part, int count, bool global) {
     double acc = 0.0;
-    for (int i = threadIdx.x; i < (int)gridDim.x; i += blockDim.x) acc += __ldcg(part + i);
-    const double tot = block_sum(acc, sh);
-    if (threadIdx.x == 0) {
-        const double nr = sqrt(tot);
-        *nrm = nr;
-        if (hist) hist[slot] = nr;
-        *ticket = 0u;
-    }
+    for (int i = threadIdx.x; i < count; i += 32) acc += global ? __ldcg(part + i) : part[i];
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(kFull, acc, o);
+    return acc;
 }
 
-// y = M x (divided by *nrm_x when nrm_x is given); *nrm_y = ||y|| (and
-// hist[slot] = ||y|| when hist is given).  Blocks [0, n_long) take one of the
-// rows longer than long_thr (a list of them) each, all threads striding over
-// its entries; the other blocks take the remaining rows with kPowGroup lanes
-// per row.
-__global__ void __launch_bounds__(kPowThreads) k_power_spmv(const int* __restrict__ rp, const int* __restrict__ ci,
-                                                            const double* __restrict__ v, int rows,
-                                                            const int* __restrict__ long_rows, int n_long,
-                                                            int long_thr, const double* __restrict__ x,
-                                                            const double* __restrict__ nrm_x,
-                                                            double* __restrict__ y, double* part,
-                                                            unsigned* __restrict__ ticket, double* __restrict__ nrm_y,
-                                                            double* __restrict__ hist, int slot) {
-    __shared__ double sh[32];
-    const double nx = nrm_x ? *nrm_x : 1.0;
-    if ((int)blockIdx.x < n_long) {
-        const int i = long_rows[blockIdx.x];
-        double acc = 0.0;
-        for (int e = rp[i] + threadIdx.x; e < rp[i + 1]; e += blockDim.x) acc += v[e] * x[ci[e]];
-        const double t = block_sum(acc, sh);
-        if (threadIdx.x == 0) {
-            const double yi = !nrm_x ? t : (nx > 0.0 ? t / nx : 0.0);
-            y[i] = yi;
-            part[blockIdx.x] = yi * yi;
+// y = 2^-e M x with e the exponent of ||x|| (FWD; 0 when the norm is 0), or
+// y = M x, and the partials of its norm.
+template <bool FWD>
+__global__ void __launch_bounds__(kPowThreads, 1) k_power_spmv(const PowArgs a) {
+    constexpr int U = 4, kGroups = kPowThreads / kPowGroup, kWarps = kPowThreads / 32;
+    __shared__ double sh[kGroups];
+    __shared__ double sh_nx;
+    const int tid = threadIdx.x, lane = tid % kPowGroup, grp = tid / kPowGroup;
+    const int stride = kPowBlocks * kGroups;
+    int i = (int)blockIdx.x * kGroups + grp;
+    // entries [b, e) of a short row; none of another
+    auto bounds = [&](int r, int& b, int& e) {
+        b = r < a.rows ? __ldg(a.rp + r) : 0;
+        e = r < a.rows ? __ldg(a.rp + r + 1) : 0;
+        if (e - b > kLongRow) e = b;
+    };
+    auto load = [&](int e0, int step, int end, int (&c)[U], double (&w)[U]) {
+#pragma unroll
+        for (int k = 0; k < U; ++k) {
+            const int e = e0 + k * step;
+            c[k] = e < end ? __ldg(a.ci + e) : -1;
+            w[k] = e < end ? __ldg(a.v + e) : 0.0;
         }
-        finish_norm(part, ticket, nrm_y, hist, slot, sh);
-        return;
+    };
+    // x was written by the previous launch: read through L2
+    auto gather = [&](const int (&c)[U], double (&xs)[U]) {
+#pragma unroll
+        for (int k = 0; k < U; ++k) xs[k] = c[k] >= 0 ? __ldcg(a.x + c[k]) : 0.0;
+    };
+    int beg, end, nbeg, nend, c[U];
+    double w[U];
+    bounds(i, beg, end);
+    load(beg + lane, kPowGroup, end, c, w);
+    bounds(i + stride, nbeg, nend);
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (*(volatile const int*)a.stop) return;
+    if (tid < 32 && (FWD || blockIdx.x == 0)) {
+        const double nx = sqrt(warp_sum(a.pin, kPowBlocks, true));
+        if (tid == 0) sh_nx = nx;
+        if (tid == 0 && blockIdx.x == 0) {
+            if (FWD) {
+                *a.xnorm = nx * pow2_below(nx);
+                // product it - 1 is complete
+                const int p = a.it - 1;
+                const double now = p > 1 ? __ldcg(a.est + p) : 0.0, before = p > 1 ? __ldcg(a.est + p - 1) : 0.0;
+                if (p >= 1 && (!(nx > 0.0) || (p > 1 && fabs(now - before) <= a.tol * now))) *a.stop = p;
+            } else {
+                const double xn = __ldcg(a.xnorm);
+                a.est[a.it] = xn > 0.0 ? nx / xn : 0.0;
+            }
+        }
     }
-    constexpr int kRowsPerWarp = 32 / kPowGroup;
-    const int lane = threadIdx.x % kPowGroup, sub = (threadIdx.x & 31) / kPowGroup;
-    const int warp = (((int)blockIdx.x - n_long) * blockDim.x + threadIdx.x) >> 5;
-    const int warps = (((int)gridDim.x - n_long) * blockDim.x) >> 5;
-    double sq = 0.0;  // the group's rows in order, in its first lane
-    // the loop bound is the same for the whole warp, so every lane reaches the shuffles
-    for (int base = warp * kRowsPerWarp; base < rows; base += warps * kRowsPerWarp) {
-        const int i = base + sub;
+    double sc = 1.0;
+    if (FWD) {
+        __syncthreads();
+        sc = sh_nx > 0.0 ? pow2_below(sh_nx) : 0.0;
+    }
+    double sq = 0.0;  // this thread's rows' squares
+    // the longest rows: a block each
+    for (int q = blockIdx.x; q < a.n_long; q += kPowBlocks) {
+        const int r = a.longs[q], b = __ldg(a.rp + r), e1 = __ldg(a.rp + r + 1);
         double acc = 0.0;
-        const bool mine = i < rows && rp[i + 1] - rp[i] <= long_thr;
-        if (mine)
-            for (int e = rp[i] + lane; e < rp[i + 1]; e += kPowGroup) acc += v[e] * x[ci[e]];
-        for (int o = kPowGroup / 2; o > 0; o >>= 1) acc += __shfl_down_sync(kFull, acc, o, kPowGroup);
-        if (lane == 0 && mine) {
-            const double yi = !nrm_x ? acc : (nx > 0.0 ? acc / nx : 0.0);
-            y[i] = yi;
+        for (int e = b + tid; e < e1; e += U * kPowThreads) {
+            int cc[U];
+            double ww[U], xs[U];
+            load(e, kPowThreads, e1, cc, ww);
+            gather(cc, xs);
+#pragma unroll
+            for (int k = 0; k < U; ++k) acc += ww[k] * xs[k];
+        }
+        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(kFull, acc, o);
+        __syncthreads();
+        if ((tid & 31) == 0) sh[tid >> 5] = acc;
+        __syncthreads();
+        if (tid < 32) {
+            const double yi = warp_sum(sh, kWarps, false) * sc;
+            if (tid == 0) {
+                a.y[r] = yi;
+                sq += yi * yi;
+            }
+        }
+    }
+    // the other long rows: a warp each
+    for (int q = (int)blockIdx.x * kWarps + (tid >> 5); q < a.n_mid; q += kPowBlocks * kWarps) {
+        const int r = a.mid[q], b = __ldg(a.rp + r), e1 = __ldg(a.rp + r + 1);
+        if (e1 - b > kPowLong) continue;
+        double acc = 0.0;
+        for (int e = b + (tid & 31); e - (tid & 31) < e1; e += U * 32) {
+            int cc[U];
+            double ww[U], xs[U];
+            load(e, 32, e1, cc, ww);
+            gather(cc, xs);
+#pragma unroll
+            for (int k = 0; k < U; ++k)
+                if (e - (tid & 31) + k * 32 < e1) acc += ww[k] * xs[k];
+        }
+        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(kFull, acc, o);
+        if ((tid & 31) == 0) {
+            const double yi = acc * sc;
+            a.y[r] = yi;
             sq += yi * yi;
         }
     }
-    const double t = block_sum(sq, sh);
-    if (threadIdx.x == 0) part[blockIdx.x] = t;
-    finish_norm(part, ticket, nrm_y, hist, slot, sh);
+    // the short rows: kPowGroup lanes each (the trip count is the block's, so
+    // that every lane reaches the shuffles)
+    for (int base = (int)blockIdx.x * kGroups; base < a.rows; base += stride) {
+        const int row = i, b = beg, e1 = end;
+        double xs[U], ws[U];
+        gather(c, xs);
+#pragma unroll
+        for (int k = 0; k < U; ++k) ws[k] = w[k];
+        beg = nbeg;
+        end = nend;
+        load(beg + lane, kPowGroup, end, c, w);
+        i += stride;
+        bounds(i + stride, nbeg, nend);
+        double acc = 0.0;
+#pragma unroll
+        for (int k = 0; k < U; ++k)
+            if (__any_sync(kFull, b + lane + k * kPowGroup < e1)) acc += ws[k] * xs[k];
+        for (int e = b + lane + U * kPowGroup; __any_sync(kFull, e < e1); e += U * kPowGroup) {
+            int cc[U];
+            load(e, kPowGroup, e1, cc, ws);
+            gather(cc, xs);
+#pragma unroll
+            for (int k = 0; k < U; ++k)
+                if (__any_sync(kFull, e + k * kPowGroup < e1)) acc += ws[k] * xs[k];
+        }
+        for (int o = kPowGroup / 2; o > 0; o >>= 1) acc += __shfl_down_sync(kFull, acc, o, kPowGroup);
+        if (lane == 0 && row < a.rows && __ldg(a.rp + row + 1) - __ldg(a.rp + row) <= kLongRow) {
+            const double yi = acc * sc;
+            a.y[row] = yi;
+            sq += yi * yi;
+        }
+    }
+    // squares sit in the groups' first lanes (the block's and the warps' rows
+    // in lanes that are among them)
+    __syncthreads();
+    if (lane == 0) sh[grp] = sq;
+    __syncthreads();
+    if (tid < 32) {
+        const double t = warp_sum(sh, kGroups, false);
+        if (tid == 0) a.pout[blockIdx.x] = t;
+    }
 }
 
-// *nrm = ||x|| with the same two-level fixed-order sum
-__global__ void __launch_bounds__(kPowThreads) k_power_norm(const double* __restrict__ x, int count,
-                                                            double* part, unsigned* __restrict__ ticket,
-                                                            double* __restrict__ nrm) {
+// partials of the squared norm of x
+__global__ void __launch_bounds__(256) k_power_norm(const double* __restrict__ x, int count, double* __restrict__ part) {
     __shared__ double sh[32];
     double acc = 0.0;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < count; i += gridDim.x * blockDim.x) acc += x[i] * x[i];
     const double t = block_sum(acc, sh);
     if (threadIdx.x == 0) part[blockIdx.x] = t;
-    finish_norm(part, ticket, nrm, nullptr, 0, sh);
 }
 
 // Blocks of the Ruiz and Pock-Chambolle row statistics (a warp per row, so
@@ -905,105 +991,99 @@ cudaError_t rhs_norm2(const double* ls, const double* us, int m, double* out_dev
     return cudaFreeAsync(part, s);
 }
 
-// (at most nnz / kLongSeg rows have more than kLongSeg entries: one block
-// and one norm partial each)
-size_t power_work_doubles(int m, int n, long long nnz, int max_iter) {
-    return (size_t)n + (size_t)(m > 0 ? m : 1) + (size_t)kPowBlocksMax + (size_t)(nnz / kLongSeg + 1) + 3 +
-           2 * ((size_t)max_iter + 1);
+size_t power_work_doubles(int m, int n, int max_iter) {
+    return (size_t)n + (size_t)(m > 0 ? m : 1) + 2 * (size_t)kPowBlocks + 2 + ((size_t)max_iter + 1);
+}
+
+// a launch of the product as a programmatic dependent of the previous one
+static cudaError_t launch_power(void (*f)(PowArgs), const PowArgs& a, cudaStream_t s) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(kPowBlocks);
+    cfg.blockDim = dim3(kPowThreads);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, f, a);
+}
+
+// The products of power_norm; va and vat list the rows of more than kPowLong
+// entries of A~ and A~^T.  `work` as power_work_doubles lays it out: w (n), u
+// (m), the partials of ||u||^2 and ||w||^2, the scaled ||w||, the stop flag,
+// the estimates; w starts as the unnormalised start vector.
+static cudaError_t power_iterate(const Csr& a, const Csr& at, const Csr& va, const Csr& vat, int max_iter,
+                                 double tol, uint64_t seed, double* work, double* est_out, int* iters_out,
+                                 cudaStream_t s) {
+    const int m = a.rows, n = a.cols;
+    double* w = work;
+    double* u = w + n;
+    double* part_u = u + (m > 0 ? m : 1);
+    double* part_w = part_u + kPowBlocks;
+    double* xnorm = part_w + kPowBlocks;
+    int* stop = reinterpret_cast<int*>(xnorm + 1);
+    double* est = xnorm + 2;
+    cudaError_t e;
+    if ((e = cudaMemsetAsync(stop, 0, sizeof(double), s)) != cudaSuccess) return e;
+    k_power_init<<<grid_for(n, 256), 256, 0, s>>>(w, n, seed);
+    k_power_norm<<<kPowBlocks, 256, 0, s>>>(w, n, part_w);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    PowArgs fwd{a.rp,  a.ci, a.v64, m, a.long_rows, a.n_long, va.long_rows, va.n_long, w,
+                u, part_w, part_u, xnorm, est, 0, stop, tol};
+    PowArgs back{at.rp, at.ci, at.v64, n, at.long_rows, at.n_long, vat.long_rows, vat.n_long, u,
+                 w, part_u, part_w, xnorm, est, 0, stop, tol};
+    // products queued between two looks at the stop flag (those past it return at once)
+    constexpr int kChunk = 64;
+    int last = 0;
+    for (int base = 1; base <= max_iter; base += kChunk) {
+        last = base + kChunk - 1 < max_iter ? base + kChunk - 1 : max_iter;
+        for (int it = base; it <= last; ++it) {
+            // u = 2^-e A~ w, then w = A~^T u and est[it] = ||A~ w|| / ||w||
+            fwd.it = back.it = it;
+            if ((e = launch_power(k_power_spmv<true>, fwd, s)) != cudaSuccess) return e;
+            if ((e = launch_power(k_power_spmv<false>, back, s)) != cudaSuccess) return e;
+        }
+        int stopped = 0;
+        if ((e = cudaMemcpyAsync(&stopped, stop, sizeof(int), cudaMemcpyDeviceToHost, s)) != cudaSuccess) return e;
+        if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return e;
+        if (stopped) {
+            last = stopped;
+            break;
+        }
+    }
+    *iters_out = last;
+    if ((e = cudaMemcpyAsync(est_out, est + last, sizeof(double), cudaMemcpyDeviceToHost, s)) != cudaSuccess) return e;
+    return cudaStreamSynchronize(s);
 }
 
 // Power iteration on A~^T A~: sigma_est = ||A~ v|| for unit v.  Stops at the
 // first product where the estimate moves by <= tol relative, or when
-// ||A~^T A~ v|| = 0, or after max_iter products.  The host looks at the
-// history every kChunk products; products past the stopping point change
-// nothing that is returned.
-static cudaError_t power_iterate(const Csr& a, const Csr& at, const Csr& va, const Csr& vat, int max_iter,
-                                 double tol, uint64_t seed, double* part, double* nrm_u, double* nrm_w,
-                                 unsigned* ticket, double* hist_est, double* hist_nw, double* w, double* u,
-                                 double* est_out, int* iters_out, cudaStream_t s);
-
+// ||A~^T A~ v|| = 0, or after max_iter products.
 cudaError_t power_norm(const Csr& a, const Csr& at, int max_iter, double tol, uint64_t seed, double* work,
                        double* est_out, int* iters_out, cudaStream_t s) {
-    const int m = a.rows, n = a.cols;
-    // work layout (power_work_doubles): w (n), u (m), part (kPowBlocksMax + nnz / kLongSeg + 1),
-    // ||u||, ||w||, the ticket, hist_est, hist_nw (max_iter + 1 each); w starts as the
-    // unnormalised start vector
-    double* w = work;
-    double* u = w + n;
-    double* part = u + (m > 0 ? m : 1);
-    double* nrm_u = part + kPowBlocksMax + (size_t)a.nnz / kLongSeg + 1;
-    double* nrm_w = nrm_u + 1;
-    unsigned* ticket = reinterpret_cast<unsigned*>(nrm_w + 1);
-    double* hist_est = nrm_w + 2;
-    double* hist_nw = hist_est + (max_iter + 1);
     cudaError_t e;
     *est_out = 0.0;
     *iters_out = 0;
-    if (m == 0 || a.nnz == 0) return cudaSuccess;
-    // the rows of more than kLongSeg entries of A~ and A~^T, one block each
+    if (a.rows == 0 || a.nnz == 0) return cudaSuccess;
+    // the rows of more than kPowLong entries of A~ and A~^T, one block each
     Csr va = a, vat = at;
     for (Csr* c : {&va, &vat}) {
+        const bool some = c->n_long > 0;  // rows of more than kLongRow entries
         c->long_rows = c->lseg = c->lseg0 = nullptr;
-        c->long_thr = kLongSeg;
-        if ((e = build_long_rows(*c, s)) != cudaSuccess) {
+        c->n_long = 0;
+        c->long_thr = kPowLong;
+        if (some && (e = build_long_rows(*c, s)) != cudaSuccess) {
             free_long_rows(va);
             free_long_rows(vat);
             return e;
         }
     }
-    e = power_iterate(a, at, va, vat, max_iter, tol, seed, part, nrm_u, nrm_w, ticket, hist_est, hist_nw, w, u,
-                      est_out, iters_out, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    e = power_iterate(a, at, va, vat, max_iter, tol, seed, work, est_out, iters_out, s);
+    if (e != cudaSuccess) cudaStreamSynchronize(s);
     free_long_rows(va);
     free_long_rows(vat);
     return e;
-}
-
-// The products of power_norm; va and vat list the rows of more than kLongSeg
-// entries of A~ and A~^T.
-static cudaError_t power_iterate(const Csr& a, const Csr& at, const Csr& va, const Csr& vat, int max_iter,
-                                 double tol, uint64_t seed, double* part, double* nrm_u, double* nrm_w,
-                                 unsigned* ticket, double* hist_est, double* hist_nw, double* w, double* u,
-                                 double* est_out, int* iters_out, cudaStream_t s) {
-    const int m = a.rows, n = a.cols;
-    cudaError_t e;
-    if ((e = cudaMemsetAsync(ticket, 0, sizeof(unsigned), s)) != cudaSuccess) return e;
-    k_power_init<<<grid_for(n, 256), 256, 0, s>>>(w, n, seed);
-    k_power_norm<<<kPowBlocks, kPowThreads, 0, s>>>(w, n, part, ticket, nrm_w);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    // products queued between two looks at the history (products past the
-    // stopping point are wasted work)
-    constexpr int kChunk = 16;
-    std::vector<double> he(kChunk), hn(kChunk);
-    double prev = -1.0;
-    for (int base = 1; base <= max_iter; base += kChunk) {
-        const int last = base + kChunk - 1 < max_iter ? base + kChunk - 1 : max_iter;
-        for (int it = base; it <= last; ++it) {
-            // u = A~ w / ||w|| (records ||u||), then w = A~^T u (records ||w||)
-            // rows of more than kLongSeg entries get a whole block each
-            k_power_spmv<<<va.n_long + pow_blocks(m), kPowThreads, 0, s>>>(a.rp, a.ci, a.v64, m, va.long_rows,
-                                                                          va.n_long, kLongSeg, w, nrm_w, u, part,
-                                                                          ticket, nrm_u, hist_est, it);
-            k_power_spmv<<<vat.n_long + pow_blocks(n), kPowThreads, 0, s>>>(at.rp, at.ci, at.v64, n, vat.long_rows,
-                                                                           vat.n_long, kLongSeg, u, nullptr, w, part,
-                                                                           ticket, nrm_w, hist_nw, it);
-        }
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        const int cnt = last - base + 1;
-        if ((e = cudaMemcpyAsync(he.data(), hist_est + base, sizeof(double) * cnt, cudaMemcpyDeviceToHost, s)) != cudaSuccess) return e;
-        if ((e = cudaMemcpyAsync(hn.data(), hist_nw + base, sizeof(double) * cnt, cudaMemcpyDeviceToHost, s)) != cudaSuccess) return e;
-        if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return e;
-        for (int q = 0; q < cnt; ++q) {
-            const int it = base + q;
-            const double est = he[q];
-            *est_out = est;
-            *iters_out = it;
-            if (!(hn[q] > 0.0)) return cudaSuccess;
-            if (prev >= 0.0 && fabs(est - prev) <= tol * est) return cudaSuccess;
-            prev = est;
-        }
-    }
-    return cudaSuccess;
 }
 
 }  // namespace lpb
