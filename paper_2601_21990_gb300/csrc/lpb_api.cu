@@ -62,6 +62,16 @@ struct lpb_batch {
 
 namespace {
 
+// the batch's points, one block: x (n per LP), then y (m per LP); each LP's
+// are written when it finishes
+cudaError_t batch_points(lpb_batch* bt) {
+    const size_t k = bt->num_lps > 0 ? bt->num_lps : 1, ny = (size_t)(bt->m > 0 ? bt->m : 1) * k;
+    const size_t nx = ((size_t)bt->n * k + 31) / 32 * 32;  // y begins on 256 bytes, as x does
+    const cudaError_t e = cudaMalloc((void**)&bt->x, sizeof(double) * (nx + ny));
+    if (e == cudaSuccess) bt->y = bt->x + nx;
+    return e;
+}
+
 template <typename T> constexpr int prec_of() {
     return std::is_same<T, float>::value ? kPrecF32 : std::is_same<T, double>::value ? kPrecF64 : kPrecDfl;
 }
@@ -141,10 +151,7 @@ lpb_err solve_impl(lpb_ctx* h, int num_lps, const lpb_lp_spec* specs_dev, double
     if ((rc = lane_reserve(h, ln, prec_of<T>(), num_lps, 1)) != LPB_OK) return rc;
     if ((rc = ensure_check_ws(h, ln.cap)) != LPB_OK) return rc;
     if ((rc = ensure_events(h)) != LPB_OK) return rc;
-    CU(cudaMalloc((void**)&bt->x, sizeof(double) * (size_t)n * (num_lps ? num_lps : 1)));
-    CU(cudaMalloc((void**)&bt->y, sizeof(double) * (size_t)(m ? m : 1) * (num_lps ? num_lps : 1)));
-    CU(cudaMemsetAsync(bt->x, 0, sizeof(double) * (size_t)n * num_lps, s));
-    CU(cudaMemsetAsync(bt->y, 0, sizeof(double) * (size_t)m * num_lps, s));
+    CU(batch_points(bt));
     bt->res.assign(num_lps, lpb_lp_result{});
     lpb_profile& prof = bt->prof;
     prof.setup_ms = h->setup_ms;
@@ -296,11 +303,7 @@ lpb_err solve_joint_impl(const std::vector<lpb_ctx*>& hs, const int32_t* num_lps
         const int nl = num_lps[i], n = h->n, m = h->m;
         if ((rc = lane_reserve(h, ln, prec, nl, 1)) != LPB_OK) break;
         if ((rc = ensure_check_ws(h, ln.cap)) != LPB_OK) break;
-        cudaError_t e = cudaMalloc((void**)&bt->x, sizeof(double) * (size_t)n * (nl ? nl : 1));
-        if (e == cudaSuccess) e = cudaMalloc((void**)&bt->y, sizeof(double) * (size_t)(m ? m : 1) * (nl ? nl : 1));
-        if (e == cudaSuccess) e = cudaMemsetAsync(bt->x, 0, sizeof(double) * (size_t)n * nl, h->stream);
-        if (e == cudaSuccess) e = cudaMemsetAsync(bt->y, 0, sizeof(double) * (size_t)m * nl, h->stream);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+        cudaError_t e = batch_points(bt);
         if (e != cudaSuccess) {
             rc = cuda_fail(e, "joint solve: result buffers");
             break;
@@ -320,6 +323,8 @@ lpb_err solve_joint_impl(const std::vector<lpb_ctx*>& hs, const int32_t* num_lps
         bt->prof.kernels += 3;
         admitted[i] = 1;
         rc = lane_admit<T>(h, ln, gi, specs_dev[i], nullptr, nullptr, n, m, tol, h->stream, groups[i]);
+        // the joint intervals run on another stream
+        if (rc == LPB_OK && (e = cudaStreamSynchronize(h->stream)) != cudaSuccess) rc = cuda_fail(e, "joint solve");
         can_stall[i] = std::is_same<T, float>::value && polish_enabled(h);
     }
     std::vector<int> all;
@@ -1006,8 +1011,7 @@ lpb_err lpb_scaling(lpb_handle h, double* d_row, double* d_col) {
 void lpb_batch_free(lpb_batch_t b) {
     if (!b) return;
     DeviceGuard guard(b->device);
-    if (b->x) cudaFree(b->x);
-    if (b->y) cudaFree(b->y);
+    if (b->x) cudaFree(b->x);  // y lies behind it
     delete b;
 }
 

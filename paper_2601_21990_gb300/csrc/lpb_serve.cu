@@ -132,8 +132,6 @@ lpb_err admit(Matrix& M, Request& r, int gid, int slot0, const double* warm_src_
     LPB_CU(cudaMemcpyAsync(r.specs_dev, r.specs.data(), sizeof(lpb_lp_spec) * r.count, cudaMemcpyHostToDevice, s));
     LPB_CU(cudaMallocAsync((void**)&r.x_dev, sizeof(double) * (size_t)n * r.count, s));
     LPB_CU(cudaMallocAsync((void**)&r.y_dev, sizeof(double) * (size_t)(m > 0 ? m : 1) * r.count, s));
-    LPB_CU(cudaMemsetAsync(r.x_dev, 0, sizeof(double) * (size_t)n * r.count, s));
-    LPB_CU(cudaMemsetAsync(r.y_dev, 0, sizeof(double) * (size_t)(m > 0 ? m : 1) * r.count, s));
     const double *wx = nullptr, *wy = nullptr;
     int64_t wsx = n, wsy = m;
     if (!r.warm_x.empty()) {

@@ -116,3 +116,28 @@ def test_steps_match_plain_iterations(lpb, precision, m, n, longest, lps):
             assert np.abs(y - ey[q]).max() <= 4000 * u * max(1.0, np.abs(ey[q] / dr).max()) * dr.max(), q
         b.free()
     h.close()
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("lps", [7, 8, 31, 33, 40])
+def test_points_of_many_columns_equal_those_of_one(lpb, precision, lps):
+    """A batch's points, extracted together (tiles from 8 columns on), are bit
+    for bit those of each LP solved alone (one column); an LP with an empty
+    box among them has zeros.  One check, so no restart couples the LPs."""
+    lp = _lp(130, 97, 6, 3)
+    sp = _specs(lp, lps, lps)
+    sp.kind[3], sp.lo[3], sp.hi[3] = 1, 5.0, 4.0  # an empty box
+    specs = lpb.specs_array(sp.kind, sp.var, sp.lo, sp.hi, sp.sign)
+    h = lpb.Handle(lp, precision=lpb.FP64 if precision == "fp64" else lpb.MIXED)
+    b = h.solve(specs, tol=1e-12, max_iter=64)
+    for q in range(lps):
+        r, x, y = b.result(q)
+        if q == 3:
+            assert r.status == lpb.PRIMAL_INFEASIBLE and not x.any() and not y.any()
+            continue
+        one = h.solve(specs[q:q + 1], tol=1e-12, max_iter=64)
+        _, x1, y1 = one.result(0)
+        assert np.array_equal(x, x1) and np.array_equal(y, y1), q
+        one.free()
+    b.free()
+    h.close()
