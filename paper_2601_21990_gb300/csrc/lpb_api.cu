@@ -450,6 +450,8 @@ lpb_err pack_rows(lpb_ctx* h, Csr& c) {
 
 lpb_err apply_shape(lpb_ctx* h, Csr& c, int thr, int shift) {
     if (c.long_thr != thr) {
+        CU(cudaStreamSynchronize(h->stream));
+        free_res_plans(h);  // laid out for the old threshold
         c.long_thr = thr;
         CU(build_long_rows(c, h->stream));
         lpb_err rc = pack_rows(h, c);
@@ -1021,6 +1023,7 @@ void lpb_destroy(lpb_handle h) {
     if (h->stream) cudaStreamSynchronize(h->stream);
     for (cudaEvent_t e : h->events) cudaEventDestroy(e);
     for (auto& ln : h->lane) lane_free(ln);
+    free_res_plans(h);
     free_list(h->ws_allocs);
     if (h->specs_dev) cudaFree(h->specs_dev);
     free_list(h->fixed_allocs);

@@ -461,18 +461,35 @@ lpb_err queue_check(lpb_ctx* h, Lane& ln, int L, int stall_checks, cudaStream_t 
     return LPB_OK;
 }
 
-// Queues the L iterations of an interval, the check and the copies of the
-// per-column and per-group records.
+// lane ln of handle h as one part of a joint launch
 template <typename T>
-lpb_err queue_interval(lpb_ctx* h, Lane& ln, int L, int stall_checks, int uni, bool timed, cudaStream_t s) {
-    const int ld = ln.cap, ce = h->opt.check_every;
-    const IterData<T> id = iter_data<T>(h, ln);
-    const IterBufs<T> ib = iter_bufs<T>(ln);
-    const T* hal = pick<T>(ln.hal64, ln.hal32, ln.haldf);
+IterPart<T> iter_part(const lpb_ctx* h, const Lane& ln, int uni) {
+    IterPart<T> q;
+    q.d = iter_data<T>(h, ln);
+    q.b = iter_bufs<T>(ln);
+    q.ld = ln.cap;
+    q.ncol = ln.ncol;
+    q.ce = h->opt.check_every;
+    q.uni = uni;
+    q.hal = pick<T>(ln.hal64, ln.hal32, ln.haldf);
+    return q;
+}
+
+// Queues the L iterations of an interval (one launch of the resident kernel
+// when shape says so, else a primal and a dual step launch each), the check
+// and the copies of the per-column and per-group records.
+template <typename T>
+lpb_err queue_interval(lpb_ctx* h, Lane& ln, int L, int stall_checks, int uni, bool timed, const ResShape& shape,
+                       ResPlan* plan, cudaStream_t s) {
+    const IterPart<T> q = iter_part<T>(h, ln, uni);
     const bool pdl = h->opt.use_pdl != 0;
-    for (int t = 0; t < L; ++t)
-        LPB_CU(launch_iteration<T>(id, ib, ld, ln.ncol, hal, t, ce, uni, t == L - 1, pdl, s,
-                                   timed ? &h->events[3 * t] : nullptr));
+    if (shape.C > 0) {
+        LPB_CU(launch_resident<T>(&q, &plan, 1, L, shape, s));
+    } else {
+        for (int t = 0; t < L; ++t)
+            LPB_CU(launch_iteration<T>(q.d, q.b, q.ld, q.ncol, q.hal, t, q.ce, uni, t == L - 1, pdl, s,
+                                       timed ? &h->events[3 * t] : nullptr));
+    }
     return queue_check<T>(h, ln, L, stall_checks, s, timed ? &h->events[3 * L] : nullptr);
 }
 
@@ -518,19 +535,21 @@ lpb_err capture_into(cudaGraphExec_t* exec, cudaStream_t s, Q queue) {
     return LPB_OK;
 }
 
-// launches, kernels and algorithmic bytes of one interval of lane ln
+// steps, kernels and algorithmic bytes of one interval of lane ln (resident:
+// its steps ran in one launch)
 template <typename T>
-void count_interval(const lpb_ctx* h, const Lane& ln, int L, lpb_profile* prof) {
+void count_interval(const lpb_ctx* h, const Lane& ln, int L, bool resident, lpb_profile* prof) {
     if (!prof) return;
     const int m = h->m;
     for (int t = 0; t < L; ++t) {
         const bool chk = t == L - 1;
         prof->launches[0] += 1;
         prof->launches[1] += m > 0 ? 1 : 0;
-        prof->kernels += m > 0 ? 2 : 1;
+        prof->kernels += resident ? 0 : m > 0 ? 2 : 1;
         prof->bytes[0] += step_bytes(prec_of<T>(), h->nnz, m, h->n, true, chk, ln.ncol);
         prof->bytes[1] += step_bytes(prec_of<T>(), h->nnz, m, h->n, false, chk, ln.ncol);
     }
+    prof->kernels += resident ? 1 : 0;
     prof->launches[2] += m > 0 ? 2 : 1;
     prof->launches[3] += 1;
     prof->checks += 1;
@@ -544,21 +563,30 @@ lpb_err lane_interval(lpb_ctx* h, Lane& ln, int L, int stall_checks, cudaStream_
     const int ce = h->opt.check_every;
     const bool timed = prof && h->opt.profile && (int)h->events.size() >= 3 * ce + 3;
     const int uni = lane_uni(ln);
+    ResShape shape;
+    ResPlan* plan = nullptr;
+    if (!timed) {
+        Lane* lp = &ln;
+        const lpb_err rc = res_choose<T>(&h, &lp, 1, &shape, &plan);
+        if (rc != LPB_OK) return rc;
+    }
     if (!h->opt.use_graphs || timed) {
-        lpb_err rc = queue_interval<T>(h, ln, L, stall_checks, uni, timed, s);
+        lpb_err rc = queue_interval<T>(h, ln, L, stall_checks, uni, timed, shape, plan, s);
         if (rc != LPB_OK) return rc;
     } else {
         // one CUDA graph per interval shape, replayed while the shape holds;
         // a new shape updates the executable graph in place when it can
-        const GraphKey key = interval_key(h, ln, L, stall_checks, uni, (int)sizeof(T));
+        GraphKey key = interval_key(h, ln, L, stall_checks, uni, (int)sizeof(T));
+        key.res = shape.C > 0 ? plan : nullptr;
+        key.res_c = shape.C;
         if (!ln.exec || !(ln.gkey == key)) {
-            const lpb_err rc = capture_into(&ln.exec, s, [&] { return queue_interval<T>(h, ln, L, stall_checks, uni, false, s); });
+            const lpb_err rc = capture_into(&ln.exec, s, [&] { return queue_interval<T>(h, ln, L, stall_checks, uni, false, shape, plan, s); });
             if (rc != LPB_OK) return rc;
             ln.gkey = key;
         }
         LPB_CU(cudaGraphLaunch(ln.exec, s));
     }
-    count_interval<T>(h, ln, L, prof);
+    count_interval<T>(h, ln, L, shape.C > 0, prof);
     return LPB_OK;
 }
 
@@ -575,21 +603,33 @@ lpb_err joint_interval(lpb_ctx* const* hs, Lane* const* lns, const int* stall_ch
     std::vector<IterPart<T>> parts(count);
     std::vector<GraphKey> keys(count);
     for (int i = 0; i < count; ++i) {
-        const lpb_ctx* h = hs[i];
-        const Lane& ln = *lns[i];
-        IterPart<T>& q = parts[i];
-        q.d = iter_data<T>(h, ln);
-        q.b = iter_bufs<T>(ln);
-        q.ld = ln.cap;
-        q.ncol = ln.ncol;
-        q.ce = h->opt.check_every;
-        q.uni = lane_uni(ln);
-        q.hal = pick<T>(ln.hal64, ln.hal32, ln.haldf);
-        keys[i] = interval_key(h, ln, L, stall_checks[i], q.uni, (int)sizeof(T));
+        parts[i] = iter_part<T>(hs[i], *lns[i], lane_uni(*lns[i]));
+        keys[i] = interval_key(hs[i], *lns[i], L, stall_checks[i], parts[i].uni, (int)sizeof(T));
+    }
+    // the resident kernel, when it is the faster way for every kMaxParts lanes
+    std::vector<ResShape> shapes;
+    std::vector<ResPlan*> plans(count, nullptr);
+    bool resident = true;
+    for (int k = 0; k < count && resident; k += kMaxParts) {
+        ResShape shape;
+        const lpb_err rc = res_choose<T>(hs + k, lns + k, std::min(kMaxParts, count - k), &shape, &plans[k]);
+        if (rc != LPB_OK) return rc;
+        resident = shape.C > 0;
+        shapes.push_back(shape);
+    }
+    for (int i = 0; i < count && resident; ++i) {
+        keys[i].res = plans[i];
+        keys[i].res_c = shapes[i / kMaxParts].C;
     }
     const bool pdl = hs[0]->opt.use_pdl != 0;
     auto queue = [&]() -> lpb_err {
-        for (int t = 0; t < L; ++t) LPB_CU(launch_iteration_multi<T>(parts.data(), count, t, t == L - 1, pdl, s));
+        if (resident) {
+            for (int k = 0; k < count; k += kMaxParts)
+                LPB_CU(launch_resident<T>(&parts[k], &plans[k], std::min(kMaxParts, count - k), L,
+                                          shapes[k / kMaxParts], s));
+        } else {
+            for (int t = 0; t < L; ++t) LPB_CU(launch_iteration_multi<T>(parts.data(), count, t, t == L - 1, pdl, s));
+        }
         for (int i = 0; i < count; ++i) {
             const lpb_err rc = queue_check<T>(hs[i], *lns[i], L, stall_checks[i], s, nullptr);
             if (rc != LPB_OK) return rc;
@@ -614,7 +654,7 @@ lpb_err joint_interval(lpb_ctx* const* hs, Lane* const* lns, const int* stall_ch
         if (rc != LPB_OK) return rc;
     }
     jg.seen = keys;
-    for (int i = 0; i < count; ++i) count_interval<T>(hs[i], *lns[i], L, profs ? profs[i] : nullptr);
+    for (int i = 0; i < count; ++i) count_interval<T>(hs[i], *lns[i], L, resident, profs ? profs[i] : nullptr);
     return LPB_OK;
 }
 

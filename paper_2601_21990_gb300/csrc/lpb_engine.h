@@ -44,12 +44,15 @@ struct GraphKey {
     const int* long_at = nullptr;
     const void* part = nullptr;         // long-row segment scratch
     int n_long_a = -1, n_long_at = -1, thr_a = -1, thr_at = -1, shift_a = -1, shift_at = -1;
+    const void* res = nullptr;          // layout of the resident interval kernel, or null, and its
+    int res_c = 0;                      // columns per block
     bool operator==(const GraphKey& o) const {
         return ncol == o.ncol && uni == o.uni && L == o.L && stall == o.stall && ws_epoch == o.ws_epoch &&
                tsize == o.tsize && ld == o.ld && X == o.X && Y == o.Y && rec == o.rec && rec_h == o.rec_h &&
                long_a == o.long_a && long_at == o.long_at && part == o.part && n_long_a == o.n_long_a &&
                n_long_at == o.n_long_at &&
-               thr_a == o.thr_a && thr_at == o.thr_at && shift_a == o.shift_a && shift_at == o.shift_at;
+               thr_a == o.thr_a && thr_at == o.thr_at && shift_a == o.shift_a && shift_at == o.shift_at &&
+               res == o.res && res_c == o.res_c;
     }
 };
 
@@ -89,6 +92,15 @@ struct Lane {
     std::vector<int> col_lp;        // column -> LP index within its group
     std::vector<char> slot_used;    // residual slots in use
 };
+
+// Launch shape of the resident interval kernel (lpb_resident.cu): columns per
+// block (0: the step kernels run instead), its threads and dynamic shared
+// memory.
+struct ResShape {
+    int C = 0, threads = 0;
+    size_t smem = 0;
+};
+struct ResPlan;  // a matrix's layout for that kernel
 
 // Where a group's results go and how far it is.
 struct GroupRun {
@@ -137,6 +149,10 @@ struct lpb_ctx {
     int lr_cap = 0;
     void* lr_part = nullptr;
     unsigned* lr_ticket = nullptr;
+    // layouts for the resident interval kernel, by iterate type and launch
+    // shape, and host copies of the row pointers of A~^T [0] and A~ [1]
+    std::vector<lpb::ResPlan*> res_plans;
+    std::vector<int> rp_host[2];
     lpb_lp_spec* specs_dev = nullptr;
     int specs_cap = 0;
     std::vector<void*> ws_allocs;
@@ -169,6 +185,18 @@ lpb_err ensure_check_ws(lpb_ctx* h, int cap);
 lpb_err ensure_long_scratch(lpb_ctx* h, int cap, bool force);
 void free_long_scratch(lpb_ctx* h);
 lpb_err ensure_specs(lpb_ctx* h, int count);
+// The resident interval kernel for the lanes lns[0 .. count) of several
+// handles (count <= kMaxParts, one iterate type): *shape with C > 0, and each
+// lane's layout, when one launch of it can run their intervals and is the
+// faster way; C = 0 otherwise.  May allocate and synchronize: not under capture.
+template <typename T>
+lpb_err res_choose(lpb_ctx* const* hs, Lane* const* lns, int count, ResShape* shape, ResPlan** plans);
+// An interval of L iterations of every part in one launch.
+template <typename T>
+cudaError_t launch_resident(const IterPart<T>* parts, ResPlan* const* plans, int count, int L, const ResShape& shape,
+                            cudaStream_t s);
+// Frees the handle's layouts; no launch that uses them may be in flight.
+void free_res_plans(lpb_ctx* h);
 // first free run of count residual slots, or -1
 int lane_find_slots(const Lane& ln, int count);
 // a free group id, or -1

@@ -343,6 +343,13 @@ struct TileParams {
 // (mul, step_from, blend), so that every kernel that runs them gives the same
 // bits.
 //
+// The iterate of one element, rebuilt from the previous reflection:
+// X^k = k/(k+1) Xb + X^0/(k+1), weights pa and pb.
+template <typename T>
+__device__ __forceinline__ T primal_iterate(T pa, T pb, T xbar, T x0) {
+    return mad(pa, xbar, mul(pb, x0));
+}
+
 // The primal step of one element: box projection, reflection (the Halpern
 // update of Eq. mainiter is applied when the next step rebuilds its
 // iterate).  acc is the row's product.
@@ -361,11 +368,12 @@ __device__ __forceinline__ void primal_element(T x, T acc, T tau, T cj, T lo, T 
     dz = inside ? -step : s - x;
 }
 
-// The dual step of one element: row projection and Halpern update.
+// The dual step of one element: row projection and Halpern update.  ys is
+// y / sigma (over_sigma).
 template <typename T>
-__device__ __forceinline__ void dual_element(T ca, T cb, T y, T y0, T acc, T sg, T isg, T lr, T ur, T& yh, T& yn,
+__device__ __forceinline__ void dual_element(T ca, T cb, T y, T ys, T y0, T acc, T sg, T lr, T ur, T& yh, T& yn,
                                              T& dz) {
-    const T s = over_sigma(y, sg, isg) + acc;
+    const T s = ys + acc;
     T p = s < ur ? s : ur;
     p = p > lr ? p : lr;
     yh = sg * (s - p);
@@ -409,7 +417,7 @@ __device__ __forceinline__ void primal_epilogue(const StepArgs<T>& a, const Tile
     for (int v = 0; v < V; ++v) {
         const int q = q0 + v;
         const T pa = a.uni >= 0 ? upa : P.pa[q], pb = a.uni >= 0 ? upb : P.pb[q];
-        const T x = mad(pa, o.z[v], mul(pb, o.z0[v]));
+        const T x = primal_iterate(pa, pb, o.z[v], o.z0[v]);
         const int key = P.key[q];
         T cj = key < 0 ? T(0) : k.c, lo = k.lo, hi = k.hi;
         if (key == row) {
@@ -436,8 +444,8 @@ __device__ __forceinline__ void dual_epilogue(const StepArgs<T>& a, const TilePa
 #pragma unroll
     for (int v = 0; v < V; ++v) {
         const T ca = a.uni >= 0 ? uca : P.ca[q0 + v], cb = a.uni >= 0 ? ucb : P.cb[q0 + v];
-        dual_element(ca, cb, o.z[v], o.z0[v], acc[v], P.sigma[q0 + v], P.isigma[q0 + v], k.lo, k.hi, yh[v],
-                     yn[v], dz[v]);
+        const T sg = P.sigma[q0 + v], ys = over_sigma(o.z[v], sg, P.isigma[q0 + v]);
+        dual_element(ca, cb, o.z[v], ys, o.z0[v], acc[v], sg, k.lo, k.hi, yh[v], yn[v], dz[v]);
     }
     stv(a.Z + off, yn);
     if (CHECK) {

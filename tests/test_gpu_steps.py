@@ -141,3 +141,35 @@ def test_points_of_many_columns_equal_those_of_one(lpb, precision, lps):
         one.free()
     b.free()
     h.close()
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed", "polish"])
+@pytest.mark.parametrize("m,n,longest,lps", [
+    (1, 3, 1, 1), (37, 50, 9, 2), (60, 41, 32, 7), (100, 90, 60, 33), (200, 300, 40, 150), (150, 100, 300, 170),
+    (64, 700, 500, 5), (300, 200, 12, 400),
+])
+def test_resident_intervals_equal_the_steps(lpb, precision, m, n, longest, lps):
+    """Small matrices run whole intervals in one launch; timed solves
+    (profile = 1) run the step kernels.  Every result and point is bit for bit
+    the same: one, two and four columns a block, ragged tiles, empty and long
+    rows, boxes and objectives, several intervals and a short last one."""
+    lp = _lp(m, n, longest, m + lps)
+    sp = _specs(lp, lps, lps)
+    specs = lpb.specs_array(sp.kind, sp.var, sp.lo, sp.hi, sp.sign)
+    opts = dict(precision=lpb.FP64 if precision == "fp64" else lpb.MIXED)
+    if precision == "polish":
+        opts["polish_stall_checks"] = 1
+    got = []
+    for profile in (0, 1):
+        h = lpb.Handle(lp, profile=profile, **opts)
+        for _ in range(2 - profile):  # a captured interval and its replay
+            b = h.solve(specs, tol=1e-9, max_iter=200)
+            kernels, steps = b.profile().kernels, sum(b.profile().launches[:2])
+            got.append([b.results()] + [v for q in range(lps) for v in b.result(q)[1:]])
+            b.free()
+        assert kernels > steps if profile else lp.nnz == 0 or lp.nnz > 1500 or kernels < steps, (kernels, steps)
+        h.close()
+    for other in got[1:]:
+        assert all(np.array_equal(x, y, equal_nan=x.dtype.kind == "f") if x.dtype.names is None
+                   else all(np.array_equal(x[f], y[f], equal_nan=x[f].dtype.kind == "f") for f in x.dtype.names)
+                   for x, y in zip(got[0], other))
