@@ -224,13 +224,16 @@ lpb_err lane_interval(lpb_ctx* h, Lane& ln, int L, int stall_checks, cudaStream_
 struct JointGraph {
     cudaGraphExec_t exec = nullptr;
     std::vector<GraphKey> keys, seen;
+    cudaEvent_t fork = nullptr;       // the interval's iterations
+    std::vector<cudaEvent_t> joined;  // each lane's check
 };
 void joint_graph_free(JointGraph& jg);
 
 // One interval of the lanes lns[0 .. count) of several handles at once (one
 // iterate type, the same check interval), all on stream s: L iterations
 // whose primal and dual steps each run as one launch over every lane
-// (launch_iteration_multi), then each lane's check and record copies.  With
+// (launch_iteration_multi, or the resident kernel), then the lanes' checks and
+// record copies side by side on the handles' own streams.  With
 // the first handle's use_graphs it is one CUDA graph in jg, replayed while
 // every lane's interval key holds (captured once a shape has held for one
 // interval).  Each lane's results are those of lane_interval on its own.

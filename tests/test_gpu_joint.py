@@ -138,6 +138,25 @@ def test_joint_solve_over_more_than_one_launch_of_parts(lpb, graphs, pdl):
         assert_same(lpb, a, j)
 
 
+@pytest.mark.parametrize("graphs", [1, 0])
+def test_joint_solve_with_a_callers_stream(lpb, graphs):
+    """The checks run on the handles' own streams; a handle on a stream of the
+    caller's (second or first, then all of the joint solve's) has its check on
+    the joint solve's stream: bitwise as alone either way."""
+    import torch
+
+    ws = [lpgen.sb_small(seed=s) for s in range(3)]
+    own = [lpb.Handle(w.lp, precision=lpb.MIXED, use_graphs=graphs) for w in ws]
+    alone = [h.solve(w.specs, tol=GPU_TOL, max_iter=200000) for h, w in zip(own, ws)]
+    stream = torch.cuda.Stream()
+    given = lpb.Handle(ws[1].lp, precision=lpb.MIXED, use_graphs=graphs, cuda_stream=stream.cuda_stream)
+    for order in ([0, 1, 2], [1, 0, 2]):
+        hs = [given if i == 1 else own[i] for i in order]
+        joint = lpb.Handle.solve_multi(hs, [ws[i].specs for i in order], tol=GPU_TOL, max_iter=200000)
+        for i, j in zip(order, joint):
+            assert_same(lpb, alone[i], j)
+
+
 def test_joint_solve_with_polish(lpb):
     """Batches that stall leave the joint FP32 launches and polish together
     in joint launches on their handles' polish lanes, bitwise as alone.  Two
