@@ -245,7 +245,7 @@ lpb_err ensure_long_scratch(lpb_ctx* h, int cap, bool force) {
     h->lr_cap = 0;
     if (cap <= 0) return LPB_OK;
     const int ntix = cap / 2 + 1;
-    const size_t segs = (size_t)h->A.n_lblocks + h->At.n_lblocks;
+    const size_t segs = (size_t)h->A.n_lseg + h->At.n_lseg;
     const size_t rows = (size_t)h->A.n_long + h->At.n_long;
     if (segs > 0) {
         LPB_CU(cudaMalloc(&h->lr_part, segs * (size_t)cap * 8));
@@ -256,9 +256,9 @@ lpb_err ensure_long_scratch(lpb_ctx* h, int cap, bool force) {
     unsigned* tick = h->lr_ticket;
     for (Csr* c : {&h->A, &h->At}) {
         c->ntix = ntix;
-        c->part = c->n_lblocks > 0 ? part : nullptr;
+        c->part = c->n_lseg > 0 ? part : nullptr;
         c->ticket = c->n_long > 0 ? tick : nullptr;
-        part += (size_t)c->n_lblocks * cap * 8;
+        part += (size_t)c->n_lseg * cap * 8;
         tick += (size_t)c->n_long * ntix;
     }
     h->lr_cap = cap;

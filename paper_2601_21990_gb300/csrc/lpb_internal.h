@@ -57,6 +57,15 @@ enum Stat {
     S_RX2         // ||dx - Pi_R(dx)||^2
 };
 
+// A long-row block of the step kernels: segment `seg` of `segs` of the long
+// row (the li-th) `row`, entries [beg, end); its row's segments have the
+// places part0 .. part0 + segs - 1 in the partial-sum scratch.  One 32-byte
+// record, so that a block's chain of round trips is one before its entries.
+struct alignas(16) LongSeg {
+    int row, beg, end, li;
+    int seg, segs, part0, pad;
+};
+
 struct Csr {
     int rows = 0, cols = 0, nnz = 0;
     int* rp = nullptr;          // rows + 1
@@ -69,6 +78,7 @@ struct Csr {
     // The other rows as the step kernels take them (build_short_rows): in
     // windows sorted by length, each row's entries together, from a multiple of
     // four on, and its cost and bounds beside its record.
+    int4* nrec = nullptr;       // the same rows for one or two lanes a row: row, fours, pairs, place in srec
     int4* srec = nullptr;       // row, its first four entries (entry index / 4), pairs of entries, entries
     int n_short = 0;
     int* pci = nullptr;         // entries: columns, and values in the iterate types in use
@@ -81,14 +91,13 @@ struct Csr {
     int long_thr = kLongRow;    // rows longer than this get a whole block (tunable)
     int g_shift = 0;            // step kernels use (lanes per row from the batch width) >> g_shift
     // Step kernels cut a long row into segments of at most kStepSeg entries,
-    // one block each, listed segment-major (every row's segment 0, then every
-    // row's segment 1, ...) so that the blocks running together gather from
-    // the same range of columns.  lseg[2 b], lseg[2 b + 1]: the long row
-    // (index into long_rows) and segment of block b; the segments of long row
-    // i are lseg0[i] .. lseg0[i + 1] - 1 in the partial-sum scratch.
-    int* lseg = nullptr;
-    int* lseg0 = nullptr;
-    int n_lblocks = 0;
+    // one block each, listed segment-major (every row's last possible segment,
+    // ..., every row's segment 0) so that the blocks running together gather
+    // from the same range of columns, and a row of several segments, which
+    // ends latest, starts first.  lseg: each block's record (LongSeg); the
+    // segments of a long row have consecutive places in the partial-sum scratch.
+    LongSeg* lseg = nullptr;
+    int n_lseg = 0;
     // partial sums of multi-segment rows, [segment][ld] in the iterate type,
     // and one completion ticket per (long row, column tile), tile stride ntix
     void* part = nullptr;

@@ -45,17 +45,19 @@ __global__ void __launch_bounds__(kBlock, (MinBlocks<T, G, B>::v)) k_step(const 
 // The step with B gathers at a time; with `if_fits`, only when its blocks
 // are all resident at once (*fits).
 template <typename T, int G, int B, bool CHECK, bool PRIMAL>
-cudaError_t launch_k(const StepArgs<T>& a, bool if_fits, bool* fits, cudaStream_t s) {
+cudaError_t launch_k(StepArgs<T> a, bool if_fits, bool* fits, cudaStream_t s) {
     constexpr int V = Vec<T>::V, GPB = kBlock / G, TN = G * V;
     static std::atomic<int> shape[kShapeDevices];  // static storage: starts at 0
     int sms = 0, per_sm = 0;
-    const cudaError_t e = launch_shape(shape, k_step<T, G, B, CHECK, PRIMAL>, &sms, &per_sm);
+    const cudaError_t e = launch_shape(shape, k_step<T, G, B, CHECK, PRIMAL>, long_smem<T, G>(1, kSegPer<G>), &sms, &per_sm);
     if (e != cudaSuccess) return e;
-    const int need = (a.n_short + GPB - 1) / GPB, tiles = (a.ncol + TN - 1) / TN;
-    *fits = ((long long)a.n_lblocks + need) * tiles <= (long long)sms * per_sm;
+    a.per = long_per<G>(a.n_lseg, sms);
+    const int nlb = (a.n_lseg + a.per - 1) / a.per, need = (a.n_short + GPB - 1) / GPB, tiles = (a.ncol + TN - 1) / TN;
+    *fits = ((long long)nlb + need) * tiles <= (long long)sms * per_sm;
     if (if_fits && !*fits) return cudaSuccess;
     const int persist = need < sms * per_sm ? need : sms * per_sm;
-    return launch_with(k_step<T, G, B, CHECK, PRIMAL>, dim3(a.n_lblocks + persist, tiles), a, a.pdl != 0, s);
+    return launch_with(k_step<T, G, B, CHECK, PRIMAL>, dim3(nlb + persist, tiles),
+                       long_smem<T, G>(a.n_lseg, a.per), a, a.pdl != 0, s);
 }
 
 template <typename T, int G, bool CHECK, bool PRIMAL>

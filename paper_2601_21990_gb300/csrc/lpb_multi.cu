@@ -68,13 +68,16 @@ cudaError_t launch_multi_k(MultiStepArgs<T>& m, bool if_fits, bool* fits, bool p
     constexpr int V = Vec<T>::V, GPB = kBlock / G, TN = G * V;
     static std::atomic<int> shape[kShapeDevices];  // static storage: starts at 0
     int sms = 0, per_sm = 0;
-    const cudaError_t e = launch_shape(shape, k_step_multi<T, G, B, CHECK, PRIMAL>, &sms, &per_sm);
+    const cudaError_t e = launch_shape(shape, k_step_multi<T, G, B, CHECK, PRIMAL>, long_smem<T, G>(1, kSegPer<G>), &sms,
+                                       &per_sm);
     if (e != cudaSuccess) return e;
-    int nlb[kMaxParts], need[kMaxParts], tiles[kMaxParts];
+    int smem = 0, nlb[kMaxParts], need[kMaxParts], tiles[kMaxParts];
     for (int p = 0; p < m.nparts; ++p) {
         StepArgs<T>& a = m.part[p];
         a.pdl = pdl ? 1 : 0;
-        nlb[p] = a.n_lblocks;
+        a.per = long_per<G>(a.n_lseg, sms);
+        nlb[p] = (a.n_lseg + a.per - 1) / a.per;
+        smem = std::max(smem, long_smem<T, G>(a.n_lseg, a.per));
         need[p] = (a.n_short + GPB - 1) / GPB;
         tiles[p] = (a.ncol + TN - 1) / TN;
     }
@@ -83,7 +86,7 @@ cudaError_t launch_multi_k(MultiStepArgs<T>& m, bool if_fits, bool* fits, bool p
     // (a part is cut to a wave of blocks only where it alone exceeds one)
     *fits = total < (long long)sms * per_sm;
     if (total == 0 || (if_fits && !*fits)) return cudaSuccess;
-    return launch_with(k_step_multi<T, G, B, CHECK, PRIMAL>, dim3((unsigned)total), m, pdl, s);
+    return launch_with(k_step_multi<T, G, B, CHECK, PRIMAL>, dim3((unsigned)total), smem, m, pdl, s);
 }
 
 template <typename T, int G, bool CHECK, bool PRIMAL>

@@ -196,10 +196,11 @@ __global__ void k_long_flags(const int* __restrict__ rp, int rows, int thr, int*
         flag[i] = (rp[i + 1] - rp[i]) > thr ? 1 : 0;
 }
 
-__global__ void k_long_lengths(const int* __restrict__ rp, const int* __restrict__ rows, int count,
-                               int* __restrict__ len) {
+// each long row with its entries' range
+__global__ void k_long_ranges(const int* __restrict__ rp, const int* __restrict__ rows, int count,
+                              int4* __restrict__ out) {
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < count; i += gridDim.x * blockDim.x)
-        len[i] = rp[rows[i] + 1] - rp[rows[i]];
+        out[i] = make_int4(rows[i], rp[rows[i]], rp[rows[i] + 1], 0);
 }
 
 __global__ void k_long_scatter(const int* __restrict__ flag, const int* __restrict__ pos, int rows,
@@ -214,9 +215,15 @@ __global__ void k_long_scatter(const int* __restrict__ flag, const int* __restri
 // Windows of kWindow rows, each sorted by length, longest first: the row
 // groups of a warp then take rows of about the same length, and rows that lie
 // near one another stay near (a window's rows share what they gather in L2).
-constexpr int kWindow = 2048;
+// Row groups of one or two lanes take the rows from a second list, of windows
+// of kNarrow rows, which a block or two takes at once: their points' sixteen or
+// 32 bytes a row are whole lines only together (256 iterations of 2 LPs on
+// 200k x 400k: 19.6 ms in the one order, 17.5 in the other; of 2 LPs on 20k x
+// 50k: 4.3 and 3.8; 16 columns and more lose up to 13% by the shorter windows).
+constexpr int kWindow = 2048, kNarrow = 128;
 
 // per window: its rows of at most thr entries
+template <int kWindow>
 __global__ void __launch_bounds__(256) k_short_count(const int* __restrict__ rp, int rows, int thr,
                                                      int* __restrict__ cnt) {
     __shared__ int sum;
@@ -234,6 +241,7 @@ __global__ void __launch_bounds__(256) k_short_count(const int* __restrict__ rp,
 
 // one block per window: bitonic sort of (length, place) keys, the rows of
 // more than thr entries last; equal lengths keep their order
+template <int kWindow>
 __global__ void __launch_bounds__(1024) k_short_order(const int* __restrict__ rp, int rows, int thr,
                                                       const int* __restrict__ first, int4* __restrict__ out) {
     __shared__ unsigned long long key[kWindow];
@@ -275,6 +283,20 @@ __global__ void k_short_place(int4* __restrict__ rec, int n, const int* __restri
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         rec[i].y = first[i];
         rec[i].z = (rec[i].w + 1) / 2;
+    }
+}
+
+// the record of each row, and the narrow list's records from it: their last
+// word is that record's place, where the row's cost and bounds stand
+__global__ void k_short_where(const int4* __restrict__ rec, int n, int* __restrict__ place) {
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) place[rec[i].x] = i;
+}
+__global__ void k_short_narrow(const int4* __restrict__ rec, const int* __restrict__ place, int n,
+                               int4* __restrict__ out) {
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+        const int p = place[out[i].x];
+        const int4 r = rec[p];
+        out[i] = make_int4(r.x, r.y, r.z, p);
     }
 }
 
@@ -740,51 +762,49 @@ cudaError_t transpose_csr(const Csr& a, const double* a_vals, Csr& at, int* perm
     return cudaFreeAsync(cnt, s);
 }
 
-// Segments of the long rows for the step kernels: long row i (length len_i)
-// gets ceil(len_i / kStepSeg) segments; blocks are listed segment-major.
+// Segments of the long rows for the step kernels: a long row of len entries
+// gets ceil(len / kStepSeg) segments of ceil(len / segments) entries, the
+// last ones shorter; blocks are listed segment-major.
 static cudaError_t build_long_segments(Csr& a, cudaStream_t s) {
     cudaError_t e;
     if (a.n_long == 0) return cudaSuccess;
-    std::vector<int> len(a.n_long);
-    int* len_dev = nullptr;
-    if ((e = cudaMallocAsync((void**)&len_dev, sizeof(int) * a.n_long, s)) != cudaSuccess) return e;
-    k_long_lengths<<<grid_for(a.n_long, 256), 256, 0, s>>>(a.rp, a.long_rows, a.n_long, len_dev);
+    std::vector<int4> rows(a.n_long);
+    int4* dev = nullptr;
+    if ((e = cudaMallocAsync((void**)&dev, sizeof(int4) * a.n_long, s)) != cudaSuccess) return e;
+    k_long_ranges<<<grid_for(a.n_long, 256), 256, 0, s>>>(a.rp, a.long_rows, a.n_long, dev);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    if ((e = cudaMemcpyAsync(len.data(), len_dev, sizeof(int) * a.n_long, cudaMemcpyDeviceToHost, s)) !=
-        cudaSuccess)
+    if ((e = cudaMemcpyAsync(rows.data(), dev, sizeof(int4) * a.n_long, cudaMemcpyDeviceToHost, s)) != cudaSuccess)
         return e;
-    if ((e = cudaFreeAsync(len_dev, s)) != cudaSuccess) return e;
+    if ((e = cudaFreeAsync(dev, s)) != cudaSuccess) return e;
     if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return e;
-    std::vector<int> seg0(a.n_long + 1, 0);
-    int max_ns = 0;
+    std::vector<int> part0(a.n_long + 1, 0);
+    int most = 0;
     for (int i = 0; i < a.n_long; ++i) {
-        const int ns = std::max(1, (len[i] + kStepSeg - 1) / kStepSeg);
-        seg0[i + 1] = seg0[i] + ns;
-        max_ns = std::max(max_ns, ns);
+        const int segs = std::max(1, (rows[i].z - rows[i].y + kStepSeg - 1) / kStepSeg);
+        part0[i + 1] = part0[i] + segs;
+        most = std::max(most, segs);
     }
-    std::vector<int> lseg;
-    lseg.reserve(2 * (size_t)seg0[a.n_long]);
-    for (int sg = 0; sg < max_ns; ++sg)
-        for (int i = 0; i < a.n_long; ++i)
-            if (sg < seg0[i + 1] - seg0[i]) {
-                lseg.push_back(i);
-                lseg.push_back(sg);
-            }
-    a.n_lblocks = seg0[a.n_long];
-    if ((e = cudaMalloc((void**)&a.lseg, sizeof(int) * lseg.size())) != cudaSuccess) return e;
-    if ((e = cudaMalloc((void**)&a.lseg0, sizeof(int) * seg0.size())) != cudaSuccess) return e;
-    if ((e = cudaMemcpy(a.lseg, lseg.data(), sizeof(int) * lseg.size(), cudaMemcpyHostToDevice)) != cudaSuccess)
-        return e;
-    return cudaMemcpy(a.lseg0, seg0.data(), sizeof(int) * seg0.size(), cudaMemcpyHostToDevice);
+    std::vector<LongSeg> lseg;
+    lseg.reserve((size_t)part0[a.n_long]);
+    for (int seg = most - 1; seg >= 0; --seg)
+        for (int i = 0; i < a.n_long; ++i) {
+            const int segs = part0[i + 1] - part0[i];
+            if (seg >= segs) continue;
+            const int each = (rows[i].z - rows[i].y + segs - 1) / segs;
+            const int beg = std::min(rows[i].z, rows[i].y + seg * each), end = std::min(rows[i].z, beg + each);
+            lseg.push_back(LongSeg{rows[i].x, beg, end, i, seg, segs, part0[i], 0});
+        }
+    a.n_lseg = part0[a.n_long];
+    if ((e = cudaMalloc((void**)&a.lseg, sizeof(LongSeg) * lseg.size())) != cudaSuccess) return e;
+    return cudaMemcpy(a.lseg, lseg.data(), sizeof(LongSeg) * lseg.size(), cudaMemcpyHostToDevice);
 }
 
 void free_long_rows(Csr& a) {
     if (a.long_rows) cudaFree(a.long_rows);
     if (a.lseg) cudaFree(a.lseg);
-    if (a.lseg0) cudaFree(a.lseg0);
     a.long_rows = nullptr;
-    a.lseg = a.lseg0 = nullptr;
-    a.n_long = a.n_lblocks = 0;
+    a.lseg = nullptr;
+    a.n_long = a.n_lseg = 0;
 }
 
 cudaError_t build_long_rows(Csr& a, cudaStream_t s) {
@@ -794,7 +814,7 @@ cudaError_t build_long_rows(Csr& a, cudaStream_t s) {
         free_long_rows(a);
     }
     a.n_long = 0;
-    a.n_lblocks = 0;
+    a.n_lseg = 0;
     if (a.rows == 0) return cudaSuccess;
     int *flag = nullptr, *total = nullptr;
     if ((e = cudaMallocAsync((void**)&flag, sizeof(int) * ((size_t)a.rows * 2 + 1), s)) != cudaSuccess) return e;
@@ -818,7 +838,7 @@ cudaError_t build_long_rows(Csr& a, cudaStream_t s) {
 
 void free_short_rows(Csr& a) {
     if (a.srec) cudaFree(a.srec);  // with all that lies behind it
-    a.srec = nullptr;
+    a.srec = a.nrec = nullptr;
     a.pci = nullptr;
     a.pv32 = a.pk32 = nullptr;
     a.pv64 = a.pk64 = nullptr;
@@ -848,13 +868,14 @@ cudaError_t build_short_rows(Csr& a, RowVectors<float> v32, RowVectors<double> v
         if (wanted) bytes += (size + 255) / 256 * 256;
         return at;
     };
-    const size_t at_rec = take(true, sizeof(int4) * n), at_ci = take(true, 4 * entries);
+    const size_t at_rec = take(true, sizeof(int4) * n), at_nrec = take(true, sizeof(int4) * n), at_ci = take(true, 4 * entries);
     const size_t at_v32 = take(v32.vals, 4 * entries), at_k32 = take(v32.vals, 16 * (size_t)n);
     const size_t at_v64 = take(v64.vals, 8 * entries), at_k64 = take(v64.vals, 32 * (size_t)n);
     const size_t at_vdf = take(vdf.vals, 8 * entries), at_kdf = take(vdf.vals, 32 * (size_t)n);
     char* mem = nullptr;
     if ((e = cudaMalloc((void**)&mem, bytes)) != cudaSuccess) return e;
     a.srec = (int4*)(mem + at_rec);
+    a.nrec = (int4*)(mem + at_nrec);
     a.pci = (int*)(mem + at_ci);
     if (v32.vals) {
         a.pv32 = (float*)(mem + at_v32);
@@ -868,20 +889,29 @@ cudaError_t build_short_rows(Csr& a, RowVectors<float> v32, RowVectors<double> v
         a.pvdf = (dfloat*)(mem + at_vdf);
         a.pkdf = (dfloat*)(mem + at_kdf);
     }
-    const int windows = (a.rows + kWindow - 1) / kWindow;
-    const size_t most = std::max((size_t)windows, (size_t)n);
+    const int windows = (a.rows + kWindow - 1) / kWindow, narrow = (a.rows + kNarrow - 1) / kNarrow;
+    const size_t most = std::max((size_t)a.rows, (size_t)n);
     int* cnt = nullptr;
     if ((e = cudaMallocAsync((void**)&cnt, sizeof(int) * most * 2, s)) != cudaSuccess) return e;
     int* first = cnt + most;
-    k_short_count<<<windows, 256, 0, s>>>(a.rp, a.rows, a.long_thr, cnt);
+    k_short_count<kNarrow><<<narrow, kNarrow, 0, s>>>(a.rp, a.rows, a.long_thr, cnt);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if ((e = exclusive_scan_i32(cnt, first, narrow, nullptr, s)) != cudaSuccess) return e;
+    k_short_order<kNarrow><<<narrow, kNarrow, 0, s>>>(a.rp, a.rows, a.long_thr, first, a.nrec);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    k_short_count<kWindow><<<windows, 256, 0, s>>>(a.rp, a.rows, a.long_thr, cnt);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if ((e = exclusive_scan_i32(cnt, first, windows, nullptr, s)) != cudaSuccess) return e;
-    k_short_order<<<windows, 1024, 0, s>>>(a.rp, a.rows, a.long_thr, first, a.srec);
+    k_short_order<kWindow><<<windows, 1024, 0, s>>>(a.rp, a.rows, a.long_thr, first, a.srec);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     k_short_fours<<<grid_for(n, 256), 256, 0, s>>>(a.srec, n, cnt);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if ((e = exclusive_scan_i32(cnt, first, n, nullptr, s)) != cudaSuccess) return e;
     k_short_place<<<grid_for(n, 256), 256, 0, s>>>(a.srec, n, first);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    k_short_where<<<grid_for(n, 256), 256, 0, s>>>(a.srec, n, cnt);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    k_short_narrow<<<grid_for(n, 256), 256, 0, s>>>(a.srec, cnt, n, a.nrec);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if ((e = cudaFreeAsync(cnt, s)) != cudaSuccess) return e;
     k_short_cols<<<grid_for((long long)n * 32, 256, kStatCap), 256, 0, s>>>(a.srec, n, a.rp, a.ci, a.pci);
@@ -1070,7 +1100,8 @@ cudaError_t power_norm(const Csr& a, const Csr& at, int max_iter, double tol, ui
     Csr va = a, vat = at;
     for (Csr* c : {&va, &vat}) {
         const bool some = c->n_long > 0;  // rows of more than kLongRow entries
-        c->long_rows = c->lseg = c->lseg0 = nullptr;
+        c->long_rows = nullptr;
+        c->lseg = nullptr;
         c->n_long = 0;
         c->long_thr = kPowLong;
         if (some && (e = build_long_rows(*c, s)) != cudaSuccess) {

@@ -45,11 +45,16 @@ template <> struct Vec<dfloat> { static constexpr int V = 2; };
 // Gathers a lane issues before it consumes them.  Four keep the registers low
 // enough for the resident warps that fill the memory pipeline.  A step of
 // fewer blocks than one wave has nothing but its rows' chains of round trips:
-// its kernels are the deep ones, eight at a time (sixteen where a row is one
-// or two lanes).  Row groups of 32 lanes have no deep kernel: a step that
-// wide and that small runs alone only for a few hundred rows.
-template <int G> constexpr int kDeep = G >= 32 ? 0 : G <= 2 ? 16 : 8;
+// its kernels are the deep ones, eight at a time (sixteen need so many
+// registers that the next step's blocks find no room to start early: 4 LPs on
+// 100k x 100k 6.6 ms a pass of 256 iterations, with eight 6.1).  Row groups of
+// 32 lanes have no deep kernel: a step that wide and that small runs alone
+// only for a few hundred rows.
+template <int G> constexpr int kDeep = G >= 32 ? 0 : 8;
 constexpr int kFlat = 4;
+
+// Row groups of at most so many lanes take the short rows from Csr::nrec.
+constexpr int kNarrowLanes = 2;
 
 template <typename T, int G, int B> struct MinBlocks {
     static constexpr int v = B > kFlat                       ? (B > 8 ? 3 : LPB_STEP_MIN_BLOCKS_DEEP)
@@ -190,6 +195,28 @@ __device__ __forceinline__ void gather_range(const int* __restrict__ ci, const T
     }
 }
 
+// the same from shared memory
+template <typename T, int V, int G, int B>
+__device__ __forceinline__ void gather_held(const int* ci, const T* va, const char* src, unsigned pitch, int beg,
+                                            int end, T (&acc)[V]) {
+#pragma unroll 1
+    for (int e = beg; e < end; e += B) {
+        T w[B], xs[B][V];
+        const int first = beg + (e - beg) / kRound<G> * kRound<G>;
+#pragma unroll
+        for (int j = 0; j < B; ++j) {
+            const bool in = e + j < end;
+            const unsigned c = (unsigned)ci[in ? e + j : first];
+            w[j] = in ? va[e + j] : T(0);
+            ldg_v(reinterpret_cast<const T*>(src + (size_t)c * pitch), xs[j]);
+        }
+#pragma unroll
+        for (int j = 0; j < B; ++j)
+#pragma unroll
+            for (int v = 0; v < V; ++v) acc[v] = dot_acc(w[j], xs[j][v], acc[v]);
+    }
+}
+
 // four or two values from an address that they fill
 __device__ __forceinline__ void ldg4(const int* p, unsigned (&r)[4]) {
     const int4 u = __ldg(reinterpret_cast<const int4*>(p));
@@ -278,9 +305,8 @@ struct StepArgs {
     const T* pva;
     const T* pk;
     int n_short;
-    const int* lseg;  // long-row blocks: (long row, segment) of each, segment-major
-    const int* lseg0; // first segment of each long row; segments of row i: lseg0[i + 1] - lseg0[i]
-    int n_lblocks;
+    const LongSeg* lseg;  // long-row blocks
+    int n_lseg, per;      // segments, and how many a block takes
     T* part;          // partial sums of multi-segment rows, [segment][ld]
     unsigned* ticket; // completion count per (long row, column tile), tile stride ntix
     int ntix;
@@ -320,6 +346,28 @@ __device__ __forceinline__ bool long_row_reduce(T (&acc)[V], T* red) {
 #pragma unroll
         for (int v = 0; v < V; ++v) acc[v] += red[(g * G + lane) * V + v];
     return true;
+}
+
+// Segments of long rows that a block takes at one or two lanes a row, where
+// they are so many that a block each would be more than a wave of mostly
+// prologue (long_per): 4 for one lane, 2 for two.  Measured with a block a
+// segment and with these: 2 LPs on the 20k x 50k power-law matrix (1500
+// segments) 5.0 and 4.4 ms a pass of 256 iterations (3.7 with the rows in the
+// narrow order), 8 LPs 4.1 and 3.7; on 100k x 200k with 50 long rows (200
+// segments), 2 LPs, 6.05 and 6.4.
+template <int G> constexpr int kSegPer = G <= 2 ? 4 / G : 1;
+template <int G>
+int long_per(int segments, int sms) {
+    return kSegPer<G> > 1 && segments > 4 * sms ? kSegPer<G> : 1;
+}
+// Dynamic shared memory of a long-row block: its partial sums, a vector per
+// lane, before them (wider rows than two lanes and narrower than 32) its
+// entries.  None where the matrix has no long row: L1 keeps what is not taken.
+template <typename T, int G>
+int long_smem(int segments, int per) {
+    if (segments == 0) return 0;
+    const int sums = per * kBlock * 16, entries = G < 32 && per == 1 ? kStepSeg * (int)(sizeof(int) + sizeof(T)) : 0;
+    return sums > entries ? sums : entries;
 }
 
 template <typename T>
@@ -501,14 +549,21 @@ __device__ __forceinline__ double add(double a, double b) { return a + b; }
 __device__ __forceinline__ dfloat add(dfloat a, dfloat b) { return a + b; }
 
 // One step (primal or dual) of the iteration on one column tile.
-//   Blocks [0, n_lblocks): one segment of a long row each (at most kStepSeg
+//   The first blocks: one segment of a long row each (at most kStepSeg
 //   entries), split into contiguous pieces over the block's G-lane row groups
-//   and reduced in shared memory.  A row of one segment is finished by its
+//   and reduced in shared memory; at one or two lanes, several segments
+//   (long_per).  A row of one segment is finished by its
 //   block; for a row of several, each block stores its partial sums, and the
 //   block that completes the row (the last to take the row's ticket; no block
 //   waits) adds the partials in segment order and finishes the row, so the
 //   result does not depend on which block ends last.
-//   Blocks [n_lblocks, gx): persistent over the short rows (srec), row group
+//   What bounds a long row is its block's chain of round trips, so the chain is
+//   short: one record (LongSeg) where there were four dependent loads, and
+//   below 32 lanes the entries are in shared memory or registers before the
+//   wait (64 LPs on the 20k x 50k power-law matrix, 256 iterations: 6.45 to
+//   6.28 ms a pass; at 32 lanes, whose blocks run in many waves, the detour
+//   cost 1.6%: 101 LPs on 200k x 400k 25.8 against 26.2 ms).
+//   The other blocks: persistent over the short rows (srec), row group
 //   g taking records g, g + stride, ...; a warp's row groups take rows of
 //   about the same length (build_short_rows).
 //   What bounds a short row: its gathers move 16 G bytes an entry from L2
@@ -529,7 +584,7 @@ __device__ __forceinline__ dfloat add(dfloat a, dfloat b) { return a + b; }
 template <typename T, int G, int B, bool CHECK, bool PRIMAL>
 __device__ __forceinline__ void step_body(const StepArgs<T>& a, const int bx, const int by, const int gx) {
     constexpr int V = Vec<T>::V, GPB = kBlock / G, TN = G * V;
-    __shared__ uint4 red[kBlock];  // a long-row block's partial sums
+    extern __shared__ uint4 red[];  // a long-row block's entries, then its partial sums (long_smem)
     __shared__ TileParams<T, TN> P;
     const int tile0 = by * TN;
     for (int q = threadIdx.x; q < TN; q += kBlock) {
@@ -570,31 +625,106 @@ __device__ __forceinline__ void step_body(const StepArgs<T>& a, const int bx, co
     const bool active = col0 < a.ncol;
     const unsigned gmask = G == 32 ? 0xffffffffu : (((1u << G) - 1u) << ((threadIdx.x & 31) & ~(G - 1)));
     const char* const src = reinterpret_cast<const char*>(a.src + (active ? col0 : tile0));
-    if (bx < a.n_lblocks) {
-        const int li = a.lseg[2 * bx], sg = a.lseg[2 * bx + 1];
-        const int s0 = a.lseg0[li], ns = a.lseg0[li + 1] - s0;
-        const int row = a.long_rows[li];
-        const int rb0 = a.rp[row], re0 = a.rp[row + 1];
-        const int sl = (re0 - rb0 + ns - 1) / ns;  // entries per segment
-        const int rb = min(re0, rb0 + sg * sl), re = min(re0, rb + sl);
+    const int per = kSegPer<G> > 1 ? a.per : 1, nlb = (a.n_lseg + per - 1) / per;
+    if (bx < nlb) {
+        const int st = kBlock / per, sub = threadIdx.x / st, is = bx * per + sub;  // threads of a segment
+        const bool some = is < a.n_lseg;
+        const int4* const rec = reinterpret_cast<const int4*>(a.lseg + (some ? is : bx * per));
+        const int4 r0 = __ldg(rec), r1 = __ldg(rec + 1);
+        const int row = r0.x, rb = r0.y, re = r0.z, ns = r1.y, s0 = r1.z;
         const int piece = (re - rb + GPB - 1) / GPB;
-        const int beg = min(re, rb + grp * piece), end = min(re, beg + piece);
-        __syncthreads();
-        pdl_wait(a.pdl);
         T acc[V];
 #pragma unroll
         for (int v = 0; v < V; ++v) acc[v] = T(0);
-        gather_range<T, V, G, B>(a.ci, a.va, src, pitch, beg, end, acc);
-        fin<V>(acc);
-        if (!long_row_reduce<T, V, G>(acc, reinterpret_cast<T*>(red))) return;
-        // only row group 0 (lanes 0 .. G-1 of warp 0) continues
+        if (kSegPer<G> > 1 && per > 1) {
+            constexpr int SP = kSegPer<G>, ST = kBlock / SP;
+            // a row group takes SP pieces, next to one another, of at most E
+            // entries; their columns and values come before the wait
+            constexpr int E = (kStepSeg + GPB - 1) / GPB, PC = B / E < 1 ? 1 : B / E < SP ? B / E : SP;
+            const int first = (threadIdx.x % ST) / G * SP;
+            T* const part = reinterpret_cast<T*>(red) + (size_t)sub * kBlock * V;
+            unsigned c[SP][E];
+            T w[SP][E];
+#pragma unroll
+            for (int p = 0; p < SP; ++p)
+#pragma unroll
+                for (int j = 0; j < E; ++j) {
+                    const int beg = rb + (first + p) * piece, e = beg + j;
+                    const bool in = j < piece && e < re;
+                    c[p][j] = (unsigned)__ldg(a.ci + (in ? e : beg < re ? beg : rb));
+                    w[p][j] = in ? ldg1(a.va + e) : T(0);
+                }
+            __syncthreads();
+            pdl_wait(a.pdl);
+#pragma unroll
+            for (int p0 = 0; p0 < SP; p0 += PC) {
+                // (plain loads: nothing but the wait stands before them, and
+                // the compiler moves read-only loads across it)
+                T xs[PC][E][V];
+#pragma unroll
+                for (int p = 0; p < PC; ++p)
+#pragma unroll
+                    for (int j = 0; j < E; ++j)
+                        ldv(reinterpret_cast<const T*>(src + (size_t)c[p0 + p][j] * pitch), xs[p][j]);
+#pragma unroll
+                for (int p = 0; p < PC; ++p) {
+                    const int k = first + p0 + p, left = re - rb - k * piece;
+                    T sum[V];
+#pragma unroll
+                    for (int v = 0; v < V; ++v) sum[v] = T(0);
+                    if (left > 0) {
+#pragma unroll
+                        for (int j = 0; j < E; ++j)
+#pragma unroll
+                            for (int v = 0; v < V; ++v) sum[v] = dot_acc(w[p0 + p][j], xs[p][j][v], sum[v]);
+                        if (E % 4 != 0) {  // (the last batch of four is filled up)
+#pragma unroll
+                            for (int v = 0; v < V; ++v) sum[v] = dot_acc(T(0), xs[p][0][v], sum[v]);
+                        }
+                    }
+                    fin<V>(sum);
+#pragma unroll
+                    for (int v = 0; v < V; ++v) part[(k * G + lane) * V + v] = sum[v];
+                }
+            }
+            __syncthreads();
+            if (!some || threadIdx.x % ST >= G) return;
+#pragma unroll
+            for (int v = 0; v < V; ++v) acc[v] = part[lane * V + v];
+#pragma unroll 8
+            for (int g = 1; g < GPB; ++g)
+#pragma unroll
+                for (int v = 0; v < V; ++v) acc[v] += part[(g * G + lane) * V + v];
+        } else {
+            const int beg = min(re, rb + grp * piece), end = min(re, beg + piece);
+            if constexpr (G < 32) {
+                // the segment's entries before the wait
+                T* const va = reinterpret_cast<T*>(red);
+                int* const ci = reinterpret_cast<int*>(va + kStepSeg);
+                for (int q = threadIdx.x; q < re - rb; q += kBlock) {
+                    ci[q] = __ldg(a.ci + rb + q);
+                    va[q] = ldg1(a.va + rb + q);
+                }
+                __syncthreads();
+                pdl_wait(a.pdl);
+                gather_held<T, V, G, B>(ci, va, src, pitch, beg - rb, end - rb, acc);
+                __syncthreads();
+            } else {
+                __syncthreads();
+                pdl_wait(a.pdl);
+                gather_range<T, V, G, B>(a.ci, a.va, src, pitch, beg, end, acc);
+            }
+            fin<V>(acc);
+            if (!long_row_reduce<T, V, G>(acc, reinterpret_cast<T*>(red))) return;
+        }
+        // only the segment's first row group continues
         if (ns > 1) {
-            if (active) stv_cg(a.part + (size_t)(s0 + sg) * a.ld + col0, acc);
+            if (active) stv_cg(a.part + (size_t)(s0 + r1.x) * a.ld + col0, acc);
             __threadfence();
             __syncwarp(gmask);
             unsigned last = 0;
             if (lane == 0) {
-                unsigned* t = a.ticket + (size_t)li * a.ntix + by;
+                unsigned* t = a.ticket + (size_t)r0.w * a.ntix + by;
                 last = atomicAdd(t, 1u) == (unsigned)(ns - 1);
                 if (last) *t = 0u;  // ready for the next launch
             }
@@ -619,15 +749,15 @@ __device__ __forceinline__ void step_body(const StepArgs<T>& a, const int bx, co
         return;
     }
 
-    const int stride = (gx - a.n_lblocks) * GPB;
-    int i = (bx - a.n_lblocks) * GPB + grp;
+    const int stride = (gx - nlb) * GPB;
+    int i = (bx - nlb) * GPB + grp;
     int4 rec = make_int4(0, 0, 0, 0);
     if (i < a.n_short) rec = __ldg(a.srec + i);
     __syncthreads();
     pdl_wait(a.pdl);
 #pragma unroll 1
     for (; i < a.n_short; i += stride) {
-        const int row = rec.x, first = rec.y, pairs = rec.z;
+        const int row = rec.x, first = rec.y, pairs = rec.z, place = G <= kNarrowLanes ? rec.w : i;
         if (i + stride < a.n_short) rec = __ldg(a.srec + i + stride);
         T acc[V];
 #pragma unroll
@@ -643,7 +773,7 @@ __device__ __forceinline__ void step_body(const StepArgs<T>& a, const int bx, co
         if (active) {
             const RowOwn<T, V> o = load_own<T, V, PRIMAL>(a, row, col0);
             T kk[4];
-            ldg4(a.pk + 4 * (size_t)i, kk);
+            ldg4(a.pk + 4 * (size_t)place, kk);
             const RowK<T> k{kk[0], kk[1], kk[2]};
             if (PRIMAL) primal_epilogue<T, V, TN, CHECK>(a, P, row, col0, lane * V, acc, o, k, uca, ucb);
             else dual_epilogue<T, V, TN, CHECK>(a, P, row, col0, lane * V, acc, o, k, uca, ucb);
@@ -662,10 +792,10 @@ inline int pack_shape(int sms, int per_sm) {
     return sms * 64 + per_sm;
 }
 
-// SM count and resident blocks per SM of kernel f (kBlock threads) on the
-// current device, through f's per-device cache `shape` (static storage)
+// SM count and resident blocks per SM of kernel f (kBlock threads, at most
+// smem bytes of dynamic shared memory) on the current device, through f's per-device cache `shape` (static storage)
 template <typename F>
-cudaError_t launch_shape(std::atomic<int>* shape, F f, int* sms, int* per_sm) {
+cudaError_t launch_shape(std::atomic<int>* shape, F f, int smem, int* sms, int* per_sm) {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
@@ -673,7 +803,7 @@ cudaError_t launch_shape(std::atomic<int>* shape, F f, int* sms, int* per_sm) {
     if (packed == 0) {
         int b = 0, n = 0;
         if ((e = cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-        if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, f, kBlock, 0)) != cudaSuccess) return e;
+        if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, f, kBlock, smem)) != cudaSuccess) return e;
         packed = pack_shape(n, b);
         if (dev >= 0 && dev < kShapeDevices) shape[dev].store(packed, std::memory_order_release);
     }
@@ -682,18 +812,18 @@ cudaError_t launch_shape(std::atomic<int>* shape, F f, int* sms, int* per_sm) {
     return cudaSuccess;
 }
 
-// f<<<grid, kBlock, 0, s>>>(a), as a programmatic dependent of the previous
+// f<<<grid, kBlock, smem, s>>>(a), as a programmatic dependent of the previous
 // kernel in s when pdl is set
 template <typename A>
-cudaError_t launch_with(void (*f)(A), dim3 grid, const A& a, bool pdl, cudaStream_t s) {
+cudaError_t launch_with(void (*f)(A), dim3 grid, int smem, const A& a, bool pdl, cudaStream_t s) {
     if (!pdl) {
-        f<<<grid, kBlock, 0, s>>>(a);
+        f<<<grid, kBlock, smem, s>>>(a);
         return cudaGetLastError();
     }
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = grid;
     cfg.blockDim = dim3(kBlock);
-    cfg.dynamicSmemBytes = 0;
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -746,14 +876,13 @@ StepArgs<T> step_args(bool primal, const IterData<T>& d, const IterBufs<T>& b, i
     a.va = primal ? d.at_vals : d.a_vals;
     a.long_rows = c.long_rows;
     a.n_long = c.n_long;
-    a.srec = c.srec;
+    a.srec = row_group_lanes<T>(ncol, c.g_shift) <= kNarrowLanes ? c.nrec : c.srec;
     a.pci = c.pci;
     a.pva = primal ? d.at_pv : d.a_pv;
     a.pk = primal ? d.at_pk : d.a_pk;
     a.n_short = c.n_short;
     a.lseg = c.lseg;
-    a.lseg0 = c.lseg0;
-    a.n_lblocks = c.n_lblocks;
+    a.n_lseg = c.n_lseg;
     a.part = (T*)c.part;
     a.ticket = c.ticket;
     a.ntix = c.ntix;

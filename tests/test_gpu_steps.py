@@ -119,6 +119,32 @@ def test_steps_match_plain_iterations(lpb, precision, m, n, longest, lps):
 
 
 @pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("m,n,longest,lps", [
+    (1500, 3000, 600, 1), (1500, 3000, 600, 2), (1500, 3000, 600, 3), (1500, 3000, 600, 5), (1500, 3000, 600, 8),
+    (700, 3000, 257, 4), (400, 3000, 600, 1), (5000, 900, 40, 2)])
+def test_narrow_batches_match_plain_iterations(lpb, precision, m, n, longest, lps):
+    """One and two lanes a row: long rows of more and of fewer segments than
+    four waves of SMs, the last block of segments not full, and short rows in
+    the narrow order.  A segment is cut into 64 or 128 pieces of at most four
+    entries, so k <= 4 + 127 + 2 + 5 additions follow one another in a row of
+    600, and |a||x| <= sqrt(600) times the norms; six products:
+    6 * 138 * 24.5 u < 20400 u of the largest value (FP64: times 4)."""
+    lp = _lp(m, n, longest, m + lps)
+    sp = _specs(lp, lps, lps)
+    h = lpb.Handle(lp, precision=lpb.FP64 if precision == "fp64" else lpb.MIXED)
+    dr, dc = h.scaling()
+    ex, ey = _three_iterations(lp, sp, dr, dc, h.info()[0])
+    u = 2.0 ** -53 * 4 if precision == "fp64" else 2.0 ** -24
+    b = h.solve(lpb.specs_array(sp.kind, sp.var, sp.lo, sp.hi, sp.sign), tol=1e-12, max_iter=3)
+    for q in range(lps):
+        _, x, y = b.result(q)
+        assert np.abs(x - ex[q]).max() <= 20400 * u * max(1.0, np.abs(ex[q] / dc).max()) * dc.max(), q
+        assert np.abs(y - ey[q]).max() <= 20400 * u * max(1.0, np.abs(ey[q] / dr).max()) * dr.max(), q
+    b.free()
+    h.close()
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
 @pytest.mark.parametrize("lps", [7, 8, 31, 33, 40])
 def test_points_of_many_columns_equal_those_of_one(lpb, precision, lps):
     """A batch's points, extracted together (tiles from 8 columns on), are bit
