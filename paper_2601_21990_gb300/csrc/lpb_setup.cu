@@ -11,6 +11,7 @@
 #include <vector>
 
 #include "lpb_internal.h"
+#include "lpb_row_order.h"
 
 namespace lpb {
 
@@ -239,8 +240,9 @@ __global__ void __launch_bounds__(256) k_short_count(const int* __restrict__ rp,
     if (threadIdx.x == 0) cnt[blockIdx.x] = sum;
 }
 
-// one block per window: bitonic sort of (length, place) keys, the rows of
-// more than thr entries last; equal lengths keep their order
+// one block per window: bitonic sort of the places' keys (short_key), the
+// rows of more than thr entries and the places past the last row at the end;
+// equal lengths keep their order
 template <int kWindow>
 __global__ void __launch_bounds__(1024) k_short_order(const int* __restrict__ rp, int rows, int thr,
                                                       const int* __restrict__ first, int4* __restrict__ out) {
@@ -248,9 +250,7 @@ __global__ void __launch_bounds__(1024) k_short_order(const int* __restrict__ rp
     const int base = blockIdx.x * kWindow;
     for (int q = threadIdx.x; q < kWindow; q += blockDim.x) {
         const int i = base + q;
-        const int len = i < rows ? rp[i + 1] - rp[i] : INT_MAX;
-        const unsigned desc = len <= thr ? (unsigned)(thr - len) : 0xffffffffu;
-        key[q] = (unsigned long long)desc << 32 | (unsigned)q;
+        key[q] = short_key(i < rows, i < rows ? rp[i + 1] - rp[i] : 0, thr, q);
     }
     __syncthreads();
     for (int k = 2; k <= kWindow; k <<= 1)
@@ -268,7 +268,7 @@ __global__ void __launch_bounds__(1024) k_short_order(const int* __restrict__ rp
             __syncthreads();
         }
     for (int q = threadIdx.x; q < kWindow; q += blockDim.x) {
-        if (key[q] >> 32 == 0xffffffffull) continue;
+        if (!is_short(key[q])) continue;
         const int i = base + (int)(key[q] & 0xffffffffull);
         out[first[blockIdx.x] + q] = make_int4(i, 0, 0, rp[i + 1] - rp[i]);
     }

@@ -199,3 +199,33 @@ def test_resident_intervals_equal_the_steps(lpb, precision, m, n, longest, lps):
         assert all(np.array_equal(x, y, equal_nan=x.dtype.kind == "f") if x.dtype.names is None
                    else all(np.array_equal(x[f], y[f], equal_nan=x[f].dtype.kind == "f") for f in x.dtype.names)
                    for x, y in zip(got[0], other))
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("thr", [1, 32, 2 ** 31 - 1])
+@pytest.mark.parametrize("m,n,longest,lps", [(130, 90, 60, 3), (300, 200, 60, 9), (2050, 900, 24, 40)])
+def test_steps_at_every_long_row_threshold(lpb, precision, thr, m, n, longest, lps):
+    """From a block for almost every row to none for any (the largest
+    threshold), on row counts that are no whole windows: x^ and y^ after three
+    iterations, as plain iterations give them.  Tolerance: a sum of k products,
+    k at most the longest row or column, is off by k u sqrt(k) times the norms;
+    six products: 6 k^1.5 u of the largest value; FP64 the same with its u,
+    times 4 for the oracle's own rounding."""
+    lp = _lp(m, n, longest, m + lps)
+    sp = _specs(lp, lps, lps)
+    h = lpb.Handle(lp, precision=lpb.FP64 if precision == "fp64" else lpb.MIXED, profile=1)
+    t = h.tuning()
+    t.long_row_primal = t.long_row_dual = thr
+    h.set_tuning(t)
+    assert (h.tuning().long_row_primal, h.tuning().long_row_dual) == (thr, thr)
+    dr, dc = h.scaling()
+    ex, ey = _three_iterations(lp, sp, dr, dc, h.info()[0])
+    k = max(np.diff(lp.row_ptr).max(), np.bincount(lp.col_idx, minlength=n).max())
+    tol = 6 * k ** 1.5 * (2.0 ** -53 * 4 if precision == "fp64" else 2.0 ** -24)
+    b = h.solve(lpb.specs_array(sp.kind, sp.var, sp.lo, sp.hi, sp.sign), tol=1e-12, max_iter=3)
+    for q in range(lps):
+        _, x, y = b.result(q)
+        assert np.abs(x - ex[q]).max() <= tol * max(1.0, np.abs(ex[q] / dc).max()) * dc.max(), q
+        assert np.abs(y - ey[q]).max() <= tol * max(1.0, np.abs(ey[q] / dr).max()) * dr.max(), q
+    b.free()
+    h.close()
