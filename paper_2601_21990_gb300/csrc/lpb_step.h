@@ -151,6 +151,20 @@ __device__ __forceinline__ bool is_inf(float v) { return isinf(v); }
 __device__ __forceinline__ bool is_inf(double v) { return isinf(v); }
 __device__ __forceinline__ bool is_inf(dfloat v) { return isinf(v.hi); }
 
+// A vector of the gathered block, row c.  The previous kernel of the interval
+// writes that block, and may still be writing it when this one starts: plain
+// loads, which no compiler moves ahead of the wait for that kernel (pdl_wait)
+// and which see what it wrote.  Read-only loads (ld.global.nc) are neither held
+// back by the wait nor defined for such data; the matrix, the records and the
+// bounds, which no step writes, take those.  Plain loads cost nothing: with
+// read-only ones and with these, a pass of 64 LPs on the 20k x 50k power-law
+// matrix 6.25 and 6.21 ms, 1024 LPs on 100k x 100k 59.7 and 59.9, 128 LPs on
+// 1M x 2M 125.1 and 124.9.
+template <typename T, int V>
+__device__ __forceinline__ void ld_iterate(const char* src, unsigned c, unsigned pitch, T (&r)[V]) {
+    ldv(reinterpret_cast<const T*>(src + (size_t)c * pitch), r);
+}
+
 // Entries are summed in rounds of kRound<G>; a row's last batch is filled up
 // with a factor 0 and the column of its round's first entry (no branch
 // between the gathers, and an infinite operand gives what it gives at every
@@ -171,7 +185,7 @@ __device__ __forceinline__ void gather_range(const int* __restrict__ ci, const T
         for (int j = 0; j < B; ++j) {
             const unsigned c = (unsigned)__ldg(ci + e + j);
             w[j] = ldg1(va + e + j);
-            ldg_v(reinterpret_cast<const T*>(src + (size_t)c * pitch), xs[j]);
+            ld_iterate(src, c, pitch, xs[j]);
         }
 #pragma unroll
         for (int j = 0; j < B; ++j)
@@ -186,7 +200,7 @@ __device__ __forceinline__ void gather_range(const int* __restrict__ ci, const T
             const bool in = e + j < end;
             const unsigned c = (unsigned)__ldg(ci + (in ? e + j : first));
             w[j] = in ? ldg1(va + e + j) : T(0);
-            ldg_v(reinterpret_cast<const T*>(src + (size_t)c * pitch), xs[j]);
+            ld_iterate(src, c, pitch, xs[j]);
         }
 #pragma unroll
         for (int j = 0; j < B; ++j)
@@ -208,7 +222,7 @@ __device__ __forceinline__ void gather_held(const int* ci, const T* va, const ch
             const bool in = e + j < end;
             const unsigned c = (unsigned)ci[in ? e + j : first];
             w[j] = in ? va[e + j] : T(0);
-            ldg_v(reinterpret_cast<const T*>(src + (size_t)c * pitch), xs[j]);
+            ld_iterate(src, c, pitch, xs[j]);
         }
 #pragma unroll
         for (int j = 0; j < B; ++j)
@@ -246,7 +260,7 @@ __device__ __forceinline__ void gather_batch(const unsigned (&c)[B], const T (&w
                                              T (&acc)[V]) {
     T xs[B][V];
 #pragma unroll
-    for (int j = 0; j < B; ++j) ldg_v(reinterpret_cast<const T*>(src + (size_t)c[j] * pitch), xs[j]);
+    for (int j = 0; j < B; ++j) ld_iterate(src, c[j], pitch, xs[j]);
 #pragma unroll
     for (int j = 0; j < B; ++j)
 #pragma unroll
@@ -658,14 +672,12 @@ __device__ __forceinline__ void step_body(const StepArgs<T>& a, const int bx, co
             pdl_wait(a.pdl);
 #pragma unroll
             for (int p0 = 0; p0 < SP; p0 += PC) {
-                // (plain loads: nothing but the wait stands before them, and
-                // the compiler moves read-only loads across it)
                 T xs[PC][E][V];
 #pragma unroll
                 for (int p = 0; p < PC; ++p)
 #pragma unroll
                     for (int j = 0; j < E; ++j)
-                        ldv(reinterpret_cast<const T*>(src + (size_t)c[p0 + p][j] * pitch), xs[p][j]);
+                        ld_iterate(src, c[p0 + p][j], pitch, xs[p][j]);
 #pragma unroll
                 for (int p = 0; p < PC; ++p) {
                     const int k = first + p0 + p, left = re - rb - k * piece;
