@@ -425,6 +425,8 @@ lpb_err time_steps(lpb_ctx* h, int count, int R, double* us_primal, double* us_d
 }
 
 lpb_err time_steps_any(lpb_ctx* h, int count, int R, double* up, double* ud) {
+    const lpb_err rc = rows_ready(h);
+    if (rc != LPB_OK) return rc;
     return h->opt.precision == LPB_MIXED ? time_steps<float>(h, count, R, up, ud)
                                          : time_steps<double>(h, count, R, up, ud);
 }
@@ -448,17 +450,44 @@ lpb_err pack_rows(lpb_ctx* h, Csr& c) {
     return LPB_OK;
 }
 
+// The rows of c for threshold thr: the long rows and their segments, the
+// packed short rows, and the segment scratch.  On an error nothing is laid
+// out, or (the last step) the scratch is left to the next solve.
+lpb_err lay_out_rows(lpb_ctx* h, Csr& c, int thr) {
+    c.laid_out = false;
+    c.long_thr = thr;
+    const cudaError_t e = build_long_rows(c, h->stream);
+    lpb_err rc = e == cudaSuccess ? pack_rows(h, c) : cuda_fail(e, "long rows");
+    if (rc != LPB_OK) {
+        cudaStreamSynchronize(h->stream);
+        free_long_rows(c);
+        free_short_rows(c);
+        cudaGetLastError();  // the next launch's error is its own
+        return rc;
+    }
+    c.laid_out = true;
+    rc = ensure_long_scratch(h, std::max(h->lr_cap, h->ws_cap), true);
+    if (rc != LPB_OK) cudaGetLastError();
+    return rc;
+}
+
+// A threshold change frees the old rows before it lays out the new ones (a
+// large matrix has no room for both).  When the new ones cannot be had, the
+// old ones are laid out again; when those cannot be had either, solves refuse
+// (rows_ready) until a later change succeeds.
 lpb_err apply_shape(lpb_ctx* h, Csr& c, int thr, int shift) {
-    if (c.long_thr != thr) {
+    if (!c.laid_out || c.long_thr != thr) {
         CU(cudaStreamSynchronize(h->stream));
+        h->ws_epoch += 1;   // captured intervals hold the old rows and layouts, also when this fails
         free_res_plans(h);  // laid out for the old threshold
-        c.long_thr = thr;
-        CU(build_long_rows(c, h->stream));
-        lpb_err rc = pack_rows(h, c);
-        if (rc != LPB_OK) return rc;
-        // the segment scratch follows the new long-row lists
-        rc = ensure_long_scratch(h, std::max(h->lr_cap, h->ws_cap), true);
-        if (rc != LPB_OK) return rc;
+        const int old = c.long_thr;
+        const lpb_err rc = lay_out_rows(h, c, thr);
+        if (rc != LPB_OK) {
+            const std::string why = lpb_last_error();
+            lay_out_rows(h, c, old);
+            set_last_error(why.c_str());
+            return rc;
+        }
     }
     c.g_shift = shift;
     h->ws_epoch += 1;  // captured intervals hold the old launch shapes
@@ -490,7 +519,7 @@ lpb_err check_solve_args(lpb_handle h, int32_t num_lps, const void* specs, doubl
     if (num_lps > 0 && !specs) return fail(LPB_ERR_INVALID_ARG, "specs is NULL");
     if (!(tol > 0.0) || !std::isfinite(tol)) return fail(LPB_ERR_INVALID_ARG, "tol must be positive and finite");
     if (max_iter < 1) return fail(LPB_ERR_INVALID_ARG, "max_iter must be >= 1");
-    return LPB_OK;
+    return rows_ready(h);
 }
 
 // host override records: kinds, variable indices, bounds and signs
@@ -733,6 +762,7 @@ lpb_err lpb_create(int32_t m, int32_t n, int64_t nnz, const int64_t* row_ptr, co
         for (Csr* c : {&h->A, &h->At}) {
             const lpb_err rc = pack_rows(h, *c);
             if (rc != LPB_OK) return rc;
+            c->laid_out = true;
         }
         // ||c~||, ||b~|| (w0) and the power iteration (eta)
         double* scal = nullptr;

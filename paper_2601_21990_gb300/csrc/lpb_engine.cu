@@ -155,6 +155,11 @@ lpb_err cuda_fail(cudaError_t e, const char* what) {
                 std::string(what) + ": " + cudaGetErrorString(e));
 }
 
+lpb_err rows_ready(const lpb_ctx* h) {
+    if (h->A.laid_out && h->At.laid_out) return LPB_OK;
+    return fail(LPB_ERR_OOM, "no memory was left for the matrix's rows when a threshold was changed; change it again");
+}
+
 bool polish_enabled(const lpb_ctx* h) { return h->opt.precision == LPB_MIXED && h->opt.fp64_polish; }
 bool polish_dfloat(const lpb_ctx* h) { return polish_enabled(h) && h->opt.polish_arith == LPB_POLISH_DFLOAT; }
 

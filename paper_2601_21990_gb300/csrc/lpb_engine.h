@@ -171,6 +171,9 @@ lpb_err cuda_fail(cudaError_t e, const char* what);
         if (_e != cudaSuccess) return ::lpb::cuda_fail(_e, #call); \
     } while (0)
 
+// LPB_ERR_OOM while the step kernels have no list of a matrix's rows: a
+// threshold change failed and so did laying out the old rows again
+lpb_err rows_ready(const lpb_ctx* h);
 bool polish_enabled(const lpb_ctx* h);
 bool polish_dfloat(const lpb_ctx* h);
 

@@ -89,6 +89,7 @@ struct Csr {
     double* pk64 = nullptr;
     dfloat* pkdf = nullptr;
     int long_thr = kLongRow;    // rows longer than this get a whole block (tunable)
+    bool laid_out = false;      // long_rows .. pkdf hold every row (false after a threshold change that failed)
     int g_shift = 0;            // step kernels use (lanes per row from the batch width) >> g_shift
     // Step kernels cut a long row into segments of at most kStepSeg entries,
     // one block each, listed segment-major (every row's last possible segment,

@@ -448,6 +448,8 @@ lpb_err lpb_server_attach(lpb_server_t srv, lpb_handle h, int32_t* matrix_id) {
     if (!srv || !h || !matrix_id) return fail(LPB_ERR_INVALID_ARG, "null argument");
     if (h->device != srv->device) return fail(LPB_ERR_INVALID_ARG, "handle is on another device");
     if (h->opt.precision != LPB_MIXED) return fail(LPB_ERR_INVALID_ARG, "serving runs FP32 iterates (LPB_MIXED)");
+    const lpb_err ready = rows_ready(h);
+    if (ready != LPB_OK) return ready;
     std::unique_ptr<Matrix> M(new (std::nothrow) Matrix());
     if (!M) return fail(LPB_ERR_OOM, "host allocation failed");
     M->h = h;

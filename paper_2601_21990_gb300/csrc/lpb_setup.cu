@@ -19,6 +19,19 @@ namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
 
+// scratch of one call, from the stream's pool; goes with the scope, also where
+// a later step fails
+struct StreamMem {
+    void* p = nullptr;
+    cudaStream_t s;
+    explicit StreamMem(cudaStream_t stream) : s(stream) {}
+    StreamMem(const StreamMem&) = delete;
+    StreamMem& operator=(const StreamMem&) = delete;
+    cudaError_t take(size_t bytes) { return cudaMallocAsync(&p, bytes, s); }
+    ~StreamMem() {
+        if (p) cudaFreeAsync(p, s);
+    }
+};
 
 // ---------------------------------------------------------------------------
 // exclusive scan of int32 (block = 1024 threads, 2 elements per thread)
@@ -709,11 +722,13 @@ cudaError_t exclusive_scan_i32(const int* in, int* out, int count, int* total_de
         return cudaSuccess;
     }
     const int tiles = (count + kScanTile - 1) / kScanTile;
+    StreamMem mem(s);
     int* sums = nullptr;
     int* offs = nullptr;
     cudaError_t e = cudaSuccess;
     if (tiles > 1) {
-        if ((e = cudaMallocAsync((void**)&sums, sizeof(int) * tiles * 2, s)) != cudaSuccess) return e;
+        if ((e = mem.take(sizeof(int) * (size_t)tiles * 2)) != cudaSuccess) return e;
+        sums = (int*)mem.p;
         offs = sums + tiles;
     }
     k_scan_tile<<<tiles, kScanThreads, 0, s>>>(in, out, count, sums);
@@ -727,7 +742,6 @@ cudaError_t exclusive_scan_i32(const int* in, int* out, int count, int* total_de
         k_copy_total<<<1, 1, 0, s>>>(in + count - 1, out + count - 1, total_dev);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
-    if (sums) e = cudaFreeAsync(sums, s);
     return e;
 }
 
@@ -769,13 +783,13 @@ static cudaError_t build_long_segments(Csr& a, cudaStream_t s) {
     cudaError_t e;
     if (a.n_long == 0) return cudaSuccess;
     std::vector<int4> rows(a.n_long);
-    int4* dev = nullptr;
-    if ((e = cudaMallocAsync((void**)&dev, sizeof(int4) * a.n_long, s)) != cudaSuccess) return e;
+    StreamMem mem(s);
+    if ((e = mem.take(sizeof(int4) * (size_t)a.n_long)) != cudaSuccess) return e;
+    int4* dev = (int4*)mem.p;
     k_long_ranges<<<grid_for(a.n_long, 256), 256, 0, s>>>(a.rp, a.long_rows, a.n_long, dev);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if ((e = cudaMemcpyAsync(rows.data(), dev, sizeof(int4) * a.n_long, cudaMemcpyDeviceToHost, s)) != cudaSuccess)
         return e;
-    if ((e = cudaFreeAsync(dev, s)) != cudaSuccess) return e;
     if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return e;
     std::vector<int> part0(a.n_long + 1, 0);
     int most = 0;
@@ -816,10 +830,9 @@ cudaError_t build_long_rows(Csr& a, cudaStream_t s) {
     a.n_long = 0;
     a.n_lseg = 0;
     if (a.rows == 0) return cudaSuccess;
-    int *flag = nullptr, *total = nullptr;
-    if ((e = cudaMallocAsync((void**)&flag, sizeof(int) * ((size_t)a.rows * 2 + 1), s)) != cudaSuccess) return e;
-    int* pos = flag + a.rows;
-    total = pos + a.rows;
+    StreamMem mem(s);
+    if ((e = mem.take(sizeof(int) * ((size_t)a.rows * 2 + 1))) != cudaSuccess) return e;
+    int *flag = (int*)mem.p, *pos = flag + a.rows, *total = pos + a.rows;
     k_long_flags<<<grid_for(a.rows, 256), 256, 0, s>>>(a.rp, a.rows, a.long_thr, flag);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if ((e = exclusive_scan_i32(flag, pos, a.rows, total, s)) != cudaSuccess) return e;
@@ -832,7 +845,6 @@ cudaError_t build_long_rows(Csr& a, cudaStream_t s) {
         k_long_scatter<<<grid_for(a.rows, 256), 256, 0, s>>>(flag, pos, a.rows, a.long_rows);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
-    if ((e = cudaFreeAsync(flag, s)) != cudaSuccess) return e;
     return build_long_segments(a, s);
 }
 
@@ -891,9 +903,9 @@ cudaError_t build_short_rows(Csr& a, RowVectors<float> v32, RowVectors<double> v
     }
     const int windows = (a.rows + kWindow - 1) / kWindow, narrow = (a.rows + kNarrow - 1) / kNarrow;
     const size_t most = std::max((size_t)a.rows, (size_t)n);
-    int* cnt = nullptr;
-    if ((e = cudaMallocAsync((void**)&cnt, sizeof(int) * most * 2, s)) != cudaSuccess) return e;
-    int* first = cnt + most;
+    StreamMem scratch(s);
+    if ((e = scratch.take(sizeof(int) * most * 2)) != cudaSuccess) return e;
+    int *cnt = (int*)scratch.p, *first = cnt + most;
     k_short_count<kNarrow><<<narrow, kNarrow, 0, s>>>(a.rp, a.rows, a.long_thr, cnt);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if ((e = exclusive_scan_i32(cnt, first, narrow, nullptr, s)) != cudaSuccess) return e;
@@ -913,7 +925,6 @@ cudaError_t build_short_rows(Csr& a, RowVectors<float> v32, RowVectors<double> v
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     k_short_narrow<<<grid_for(n, 256), 256, 0, s>>>(a.srec, cnt, n, a.nrec);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    if ((e = cudaFreeAsync(cnt, s)) != cudaSuccess) return e;
     k_short_cols<<<grid_for((long long)n * 32, 256, kStatCap), 256, 0, s>>>(a.srec, n, a.rp, a.ci, a.pci);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if ((e = pack_vals<float>(a, n, v32, a.pv32, a.pk32, s)) != cudaSuccess) return e;
