@@ -28,6 +28,7 @@
 #include <atomic>
 #include <climits>
 #include <cstring>
+#include <memory>
 #include <new>
 
 #include "lpb_engine.h"
@@ -410,7 +411,7 @@ __global__ void k_res_fill(ResDir<T> d, ResRec<T>* rec, Pair<T>* ova, uint32_t* 
 // row-group widths and thresholds.
 struct ResPlan {
     int prec = -1, lanes_p = 0, lanes_d = 0, thr_p = 0, thr_d = 0;
-    bool fits = false;   // laid out (else the key of a matrix that cannot be)
+    bool fits = false;   // laid out (else the key of a matrix that cannot be, or had no memory)
     int places = 0;      // rows of both products, idle lanes among them
     int slots = 0;       // partial sums (32 to a slot) of the product with more
     int slices = 0;      // slices of the longest phase
@@ -424,6 +425,7 @@ namespace {
 template <typename P>
 cudaError_t res_put(std::vector<void*>& list, const P** out, const void* src, size_t bytes, cudaStream_t s) {
     void* p = nullptr;
+    list.reserve(list.size() + 1);
     cudaError_t e = cudaMalloc(&p, bytes ? bytes : 1);
     if (e != cudaSuccess) return e;
     list.push_back(p);
@@ -449,7 +451,13 @@ lpb_err res_build(lpb_ctx* h, ResPlan* plan, long long max_pairs) {
                         lay[q]))
             return LPB_OK;
     }
-    std::vector<void*> tmp;
+    struct Staging {
+        std::vector<void*> v;
+        ~Staging() {
+            for (void* p : v) cudaFree(p);
+        }
+    } staging;
+    std::vector<void*>& tmp = staging.v;
     auto build = [&]() -> lpb_err {
         for (int q = 0; q < 2; ++q) {
             const ResLayout& l = lay[q];
@@ -490,9 +498,7 @@ lpb_err res_build(lpb_ctx* h, ResPlan* plan, long long max_pairs) {
         plan->fits = true;
         return LPB_OK;
     };
-    const lpb_err rc = build();
-    for (void* p : tmp) cudaFree(p);
-    return rc;
+    return build();
 }
 static_assert(sizeof(ResDir<float>) == sizeof(ResDir<double>) && sizeof(ResDir<dfloat>) == sizeof(ResDir<double>),
               "pointers and counts only");
@@ -542,9 +548,14 @@ cudaError_t res_launch(const ResArgs<T>& g, int threads, size_t smem, cudaStream
 
 }  // namespace
 
+static void free_res_mem(ResPlan* p) {
+    for (void* q : p->mem) cudaFree(q);
+    p->mem.clear();
+}
+
 void free_res_plans(lpb_ctx* h) {
     for (ResPlan* p : h->res_plans) {
-        for (void* q : p->mem) cudaFree(q);
+        free_res_mem(p);
         delete p;
     }
     h->res_plans.clear();
@@ -583,7 +594,8 @@ double step_us(long long pairs, bool longs, int ncol) {
 
 // The handle's layout for iterate type T (of lane precision prec) at a batch
 // width, built when there is none yet; null when the matrix has no layout of
-// at most max_pairs.
+// at most max_pairs, or no memory was left for it: the step kernels need none
+// and give the same results, so that is no error of the solve.
 template <typename T>
 lpb_err res_plan(lpb_ctx* h, int prec, int ncol, long long max_pairs, ResPlan** out) {
     *out = nullptr;
@@ -596,16 +608,27 @@ lpb_err res_plan(lpb_ctx* h, int prec, int ncol, long long max_pairs, ResPlan** 
             if (q->fits) *out = q;
             return LPB_OK;
         }
-    ResPlan* p = new (std::nothrow) ResPlan();
-    if (!p) return fail(LPB_ERR_OOM, "host allocation failed");
-    h->res_plans.push_back(p);  // no key yet: prec is -1 until it is laid out
+    std::unique_ptr<ResPlan> own(new ResPlan());
+    ResPlan* p = own.get();
+    p->prec = prec;
     p->lanes_p = lp;
     p->lanes_d = ld;
     p->thr_p = h->At.long_thr;
     p->thr_d = h->A.long_thr;
-    const lpb_err rc = res_build<T>(h, p, max_pairs);
-    if (rc != LPB_OK) return rc;
-    p->prec = prec;
+    h->res_plans.reserve(h->res_plans.size() + 1);
+    lpb_err rc = LPB_ERR_OOM;
+    try {
+        rc = res_build<T>(h, p, max_pairs);
+    } catch (const std::bad_alloc&) {
+    }
+    if (rc != LPB_OK) {
+        cudaStreamSynchronize(h->stream);
+        free_res_mem(p);
+        if (rc != LPB_ERR_OOM) return rc;
+        p->fits = false;
+        cudaGetLastError();  // the next launch's error is its own
+    }
+    h->res_plans.push_back(own.release());
     if (p->fits) *out = p;
     return LPB_OK;
 }
@@ -642,7 +665,11 @@ lpb_err res_choose(lpb_ctx* const* hs, Lane* const* lns, int count, ResShape* sh
     for (int i = 0; i < count; ++i) {
         lpb_ctx* h = hs[i];
         ResPlan* p = nullptr;
-        const lpb_err rc = res_plan<T>(h, lns[i]->prec, lns[i]->ncol, kMostPairs, &p);
+        lpb_err rc = LPB_OK;
+        try {
+            rc = res_plan<T>(h, lns[i]->prec, lns[i]->ncol, kMostPairs, &p);
+        } catch (const std::bad_alloc&) {
+        }
         if (rc != LPB_OK) return rc;
         if (!p) return LPB_OK;
         plans[i] = p;

@@ -47,6 +47,10 @@ long launches(const char* part) {
     return n;
 }
 
+bool last_error() {
+    Lock l(st().mu);
+    return st().last != cudaSuccess;
+}
 long device_waits() {
     Lock l(st().mu);
     return st().waits;

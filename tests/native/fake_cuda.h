@@ -17,6 +17,8 @@ void fail_none();
 size_t live_bytes();
 // launches so far of the kernels whose name contains `part`
 long launches(const char* part);
+// whether the runtime holds an error for cudaGetLastError
+bool last_error();
 // calls so far that wait for the whole device: cudaMalloc and cudaFree
 long device_waits();
 

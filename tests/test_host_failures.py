@@ -38,3 +38,7 @@ def _run(objects, tmp_path, name):
 
 def test_a_threshold_change_without_memory_keeps_the_rows(objects, tmp_path):
     _run(objects, tmp_path, "set_tuning_alloc_test")
+
+
+def test_a_layout_without_memory_leaves_the_step_kernels(objects, tmp_path):
+    _run(objects, tmp_path, "resident_alloc_test")
