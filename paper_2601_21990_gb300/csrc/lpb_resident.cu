@@ -407,98 +407,131 @@ __global__ void k_res_fill(ResDir<T> d, ResRec<T>* rec, Pair<T>* ova, uint32_t* 
 
 }  // namespace
 
-// A matrix's two layouts on the device, for one iterate type and set of
-// row-group widths and thresholds.
+// A matrix's two layouts for one iterate type and set of row-group widths and
+// thresholds.  Measured on the host first (measure); on the device only once
+// an interval is to run from them (res_build).
 struct ResPlan {
     int prec = -1, lanes_p = 0, lanes_d = 0, thr_p = 0, thr_d = 0;
-    bool fits = false;   // laid out (else the key of a matrix that cannot be, or had no memory)
+    bool fits = false;   // the matrix has the layouts, and no allocation for them has failed
     int places = 0;      // rows of both products, idle lanes among them
     int slots = 0;       // partial sums (32 to a slot) of the product with more
     int slices = 0;      // slices of the longest phase
     long long pairs = 0; // of a lane, both products
-    std::vector<void*> mem;
-    ResDir<double> dir[2];  // pointers; the value type follows prec
+    std::unique_ptr<ResLayout[]> lay;  // until they are on the device
+    void* mem = nullptr;               // both layouts and what they were filled from, one allocation
+    ResDir<double> dir[2];             // pointers; the value type follows prec
+    // (rp: the row pointers of A~^T, then of A~); false: no such layouts
+    bool measure(const std::vector<int>* rp, long long max_pairs) {
+        const int thr[2] = {thr_p, thr_d}, lanes[2] = {lanes_p, lanes_d};
+        lay.reset(new ResLayout[2]);
+        places = slots = slices = 0;
+        pairs = 0;
+        for (int q = 0; q < 2; ++q) {
+            ResLayout& l = lay[q];
+            if (!res_layout((int)rp[q].size() - 1, rp[q].data(), thr[q], kStepSeg, kBlock / lanes[q], max_pairs, l)) {
+                lay.reset();
+                return false;
+            }
+            places += l.places();
+            slots = std::max(slots, l.slots);
+            slices = std::max(slices, std::max(l.pieces, l.shorts + l.longs));
+            pairs += l.total_pairs;
+        }
+        return true;
+    }
 };
 
 namespace {
 
-template <typename P>
-cudaError_t res_put(std::vector<void*>& list, const P** out, const void* src, size_t bytes, cudaStream_t s) {
-    void* p = nullptr;
-    list.reserve(list.size() + 1);
-    cudaError_t e = cudaMalloc(&p, bytes ? bytes : 1);
-    if (e != cudaSuccess) return e;
-    list.push_back(p);
-    *out = (const P*)p;
-    return bytes && src ? cudaMemcpyAsync(p, src, bytes, cudaMemcpyHostToDevice, s) : cudaSuccess;
-}
+// the pieces of one allocation, each from a multiple of 256 bytes on
+struct Carve {
+    size_t bytes = 0;
+    size_t take(size_t size) {
+        const size_t at = bytes;
+        bytes += (size + 255) / 256 * 256;
+        return at;
+    }
+};
 
+// The measured layouts on the device.  The allocation is stream-ordered and
+// the only wait is for the handle's own stream: cudaMalloc and cudaFree wait
+// for the whole device, and a server runs other matrices' intervals meanwhile.
 template <typename T>
-lpb_err res_build(lpb_ctx* h, ResPlan* plan, long long max_pairs) {
+cudaError_t res_build(lpb_ctx* h, ResPlan* plan) {
     cudaStream_t s = h->stream;
     const IterData<T> it = lane_iter_data<T>(h, h->lane[0]);  // matrix and vectors only
     const Csr* csr[2] = {&h->At, &h->A};
-    const int lanes[2] = {plan->lanes_p, plan->lanes_d};
-    ResLayout lay[2];
+    struct Places {
+        size_t head, pword, lhead, np, flag, word, beg, len, pos, rec, va, ci;
+    } at[2];
+    Carve c;
     for (int q = 0; q < 2; ++q) {
-        if (h->rp_host[q].empty()) {
-            std::vector<int> rp((size_t)csr[q]->rows + 1);
-            LPB_CU(cudaMemcpyAsync(rp.data(), csr[q]->rp, sizeof(int) * rp.size(), cudaMemcpyDeviceToHost, s));
-            LPB_CU(cudaStreamSynchronize(s));
-            h->rp_host[q].swap(rp);
-        }
-        if (!res_layout(csr[q]->rows, h->rp_host[q].data(), csr[q]->long_thr, kStepSeg, kBlock / lanes[q], max_pairs,
-                        lay[q]))
-            return LPB_OK;
+        const ResLayout& l = plan->lay[q];
+        at[q].head = c.take(l.head.size() * sizeof(int2));
+        at[q].lhead = c.take(l.lhead.size() * sizeof(int4));
+        at[q].np = c.take(l.np.size() * 4);
+        at[q].flag = c.take(l.flag.size() * 4);
+        at[q].word = c.take(l.word.size() * 4);
+        at[q].pword = at[q].word + 4 * (size_t)l.places();  // the words of the piece slices are the last
+        at[q].beg = c.take(l.beg.size() * 4);
+        at[q].len = c.take(l.len.size() * 4);
+        at[q].pos = c.take(l.pos.size() * 4);
     }
-    struct Staging {
-        std::vector<void*> v;
-        ~Staging() {
-            for (void* p : v) cudaFree(p);
-        }
-    } staging;
-    std::vector<void*>& tmp = staging.v;
-    auto build = [&]() -> lpb_err {
-        for (int q = 0; q < 2; ++q) {
-            const ResLayout& l = lay[q];
-            ResDir<T> d{};
-            d.shorts = l.shorts;
-            d.longs = l.longs;
-            d.pieces = l.pieces;
-            std::vector<int> lh;
-            for (const auto& x : l.lhead) lh.insert(lh.end(), {x.pieces, x.slot0, x.flag0, 0});
-            const size_t items = 32 * (size_t)(l.shorts + l.longs), lanes32 = 32 * (size_t)l.total_pairs;
-            LPB_CU(res_put(plan->mem, &d.head, l.head.data(), l.head.size() * 8, s));
-            LPB_CU(res_put(plan->mem, &d.rec, nullptr, items * sizeof(ResRec<T>), s));
-            LPB_CU(res_put(plan->mem, &d.pword, l.word.data() + items, 4 * 32 * (size_t)l.pieces, s));
-            LPB_CU(res_put(plan->mem, &d.va, nullptr, lanes32 * sizeof(Pair<T>), s));
-            LPB_CU(res_put(plan->mem, &d.ci, nullptr, lanes32 * 4, s));
-            LPB_CU(res_put(plan->mem, &d.lhead, lh.data(), lh.size() * 4, s));
-            LPB_CU(res_put(plan->mem, &d.np, l.np.data(), l.np.size() * 4, s));
-            LPB_CU(res_put(plan->mem, &d.flag, l.flag.data(), l.flag.size() * 4, s));
-            const uint32_t* word = nullptr;
-            const int *beg = nullptr, *len = nullptr, *pos = nullptr;
-            LPB_CU(res_put(tmp, &word, l.word.data(), l.word.size() * 4, s));
-            LPB_CU(res_put(tmp, &beg, l.beg.data(), l.beg.size() * 4, s));
-            LPB_CU(res_put(tmp, &len, l.len.data(), l.len.size() * 4, s));
-            LPB_CU(res_put(tmp, &pos, lay[1 - q].pos.data(), lay[1 - q].pos.size() * 4, s));
-            const int all = 32 * (l.shorts + l.longs + l.pieces);
-            k_res_fill<T><<<(all + 127) / 128, 128, 0, s>>>(
-                d, (ResRec<T>*)d.rec, (Pair<T>*)d.va, (uint32_t*)d.ci, word, beg, len, pos, csr[q]->ci,
-                q == 0 ? it.at_vals : it.a_vals, q == 0 ? it.xl : it.l, q == 0 ? it.xu : it.u, q == 0 ? it.c : nullptr);
-            LPB_CU(cudaGetLastError());
-            LPB_CU(cudaStreamSynchronize(s));  // the staging vectors go
-            ResDir<double>& o = plan->dir[q];
-            std::memcpy((void*)&o, (const void*)&d, sizeof(o));
-            plan->places += l.places();
-            plan->slots = std::max(plan->slots, l.slots);
-            plan->slices = std::max(plan->slices, std::max(l.pieces, l.shorts + l.longs));
-            plan->pairs += l.total_pairs;
-        }
-        plan->fits = true;
-        return LPB_OK;
+    const size_t upload = c.bytes;
+    for (int q = 0; q < 2; ++q) {
+        const ResLayout& l = plan->lay[q];
+        at[q].rec = c.take((size_t)l.places() * sizeof(ResRec<T>));
+        at[q].va = c.take(32 * (size_t)l.total_pairs * sizeof(Pair<T>));
+        at[q].ci = c.take(32 * (size_t)l.total_pairs * 4);
+    }
+    std::vector<char> host(upload);
+    auto put = [&](size_t to, const void* from, size_t bytes) {
+        if (bytes) std::memcpy(host.data() + to, from, bytes);
     };
-    return build();
+    for (int q = 0; q < 2; ++q) {
+        const ResLayout& l = plan->lay[q];
+        std::vector<int4> lh;
+        for (const auto& x : l.lhead) lh.push_back(make_int4(x.pieces, x.slot0, x.flag0, 0));
+        put(at[q].head, l.head.data(), l.head.size() * sizeof(int2));
+        put(at[q].lhead, lh.data(), lh.size() * sizeof(int4));
+        put(at[q].np, l.np.data(), l.np.size() * 4);
+        put(at[q].flag, l.flag.data(), l.flag.size() * 4);
+        put(at[q].word, l.word.data(), l.word.size() * 4);
+        put(at[q].beg, l.beg.data(), l.beg.size() * 4);
+        put(at[q].len, l.len.data(), l.len.size() * 4);
+        put(at[q].pos, l.pos.data(), l.pos.size() * 4);
+    }
+    cudaError_t e;
+    if ((e = cudaMallocAsync(&plan->mem, c.bytes, s)) != cudaSuccess) return e;
+    char* mem = (char*)plan->mem;
+    if ((e = cudaMemcpyAsync(mem, host.data(), upload, cudaMemcpyHostToDevice, s)) != cudaSuccess) return e;
+    for (int q = 0; q < 2; ++q) {
+        const ResLayout& l = plan->lay[q];
+        const Places& p = at[q];
+        ResDir<T> d{};
+        d.shorts = l.shorts;
+        d.longs = l.longs;
+        d.pieces = l.pieces;
+        d.head = (const int2*)(mem + p.head);
+        d.rec = (const ResRec<T>*)(mem + p.rec);
+        d.pword = (const uint32_t*)(mem + p.pword);
+        d.va = (const Pair<T>*)(mem + p.va);
+        d.ci = (const uint32_t*)(mem + p.ci);
+        d.lhead = (const int4*)(mem + p.lhead);
+        d.np = (const int*)(mem + p.np);
+        d.flag = (const uint32_t*)(mem + p.flag);
+        const int all = 32 * (l.shorts + l.longs + l.pieces);
+        k_res_fill<T><<<(all + 127) / 128, 128, 0, s>>>(
+            d, (ResRec<T>*)d.rec, (Pair<T>*)d.va, (uint32_t*)d.ci, (const uint32_t*)(mem + p.word),
+            (const int*)(mem + p.beg), (const int*)(mem + p.len), (const int*)(mem + at[1 - q].pos), csr[q]->ci,
+            q == 0 ? it.at_vals : it.a_vals, q == 0 ? it.xl : it.l, q == 0 ? it.xu : it.u, q == 0 ? it.c : nullptr);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        std::memcpy((void*)&plan->dir[q], (const void*)&d, sizeof(d));
+    }
+    // the host's copy goes, and other streams run from the layouts
+    if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return e;
+    plan->lay.reset();
+    return cudaSuccess;
 }
 static_assert(sizeof(ResDir<float>) == sizeof(ResDir<double>) && sizeof(ResDir<dfloat>) == sizeof(ResDir<double>),
               "pointers and counts only");
@@ -548,14 +581,9 @@ cudaError_t res_launch(const ResArgs<T>& g, int threads, size_t smem, cudaStream
 
 }  // namespace
 
-static void free_res_mem(ResPlan* p) {
-    for (void* q : p->mem) cudaFree(q);
-    p->mem.clear();
-}
-
 void free_res_plans(lpb_ctx* h) {
     for (ResPlan* p : h->res_plans) {
-        free_res_mem(p);
+        if (p->mem) cudaFree(p->mem);
         delete p;
     }
     h->res_plans.clear();
@@ -592,10 +620,9 @@ double step_us(long long pairs, bool longs, int ncol) {
     return (f64 ? 6.3 : 4.3 + (longs ? 2.0 : 0.0)) + (f64 ? 2.5e-4 : 5.2e-5) * (double)pairs * ncol;
 }
 
-// The handle's layout for iterate type T (of lane precision prec) at a batch
-// width, built when there is none yet; null when the matrix has no layout of
-// at most max_pairs, or no memory was left for it: the step kernels need none
-// and give the same results, so that is no error of the solve.
+// The handle's layouts for iterate type T (of lane precision prec) at a batch
+// width, measured when they are not yet; null when the matrix has none of at
+// most max_pairs, or no memory was left for them.
 template <typename T>
 lpb_err res_plan(lpb_ctx* h, int prec, int ncol, long long max_pairs, ResPlan** out) {
     *out = nullptr;
@@ -608,28 +635,48 @@ lpb_err res_plan(lpb_ctx* h, int prec, int ncol, long long max_pairs, ResPlan** 
             if (q->fits) *out = q;
             return LPB_OK;
         }
-    std::unique_ptr<ResPlan> own(new ResPlan());
-    ResPlan* p = own.get();
+    const Csr* csr[2] = {&h->At, &h->A};
+    for (int q = 0; q < 2; ++q)
+        if (h->rp_host[q].empty()) {
+            std::vector<int> rp((size_t)csr[q]->rows + 1);
+            LPB_CU(cudaMemcpyAsync(rp.data(), csr[q]->rp, sizeof(int) * rp.size(), cudaMemcpyDeviceToHost, h->stream));
+            LPB_CU(cudaStreamSynchronize(h->stream));
+            h->rp_host[q].swap(rp);
+        }
+    std::unique_ptr<ResPlan> p(new ResPlan());
     p->prec = prec;
     p->lanes_p = lp;
     p->lanes_d = ld;
     p->thr_p = h->At.long_thr;
     p->thr_d = h->A.long_thr;
+    p->fits = p->measure(h->rp_host, max_pairs);
     h->res_plans.reserve(h->res_plans.size() + 1);
-    lpb_err rc = LPB_ERR_OOM;
+    if (p->fits) *out = p.get();
+    h->res_plans.push_back(p.release());
+    return LPB_OK;
+}
+
+// A measured plan's layouts on the device, if they are not there yet; *ok =
+// false when no memory is left for them.  The step kernels need none and give
+// the same results, so that is no error of the solve.
+template <typename T>
+lpb_err res_ready(lpb_ctx* h, ResPlan* p, long long max_pairs, bool* ok) {
+    *ok = true;
+    if (p->mem) return LPB_OK;
+    cudaError_t e = cudaErrorMemoryAllocation;
     try {
-        rc = res_build<T>(h, p, max_pairs);
+        if (p->lay || p->measure(h->rp_host, max_pairs)) e = res_build<T>(h, p);
     } catch (const std::bad_alloc&) {
     }
-    if (rc != LPB_OK) {
-        cudaStreamSynchronize(h->stream);
-        free_res_mem(p);
-        if (rc != LPB_ERR_OOM) return rc;
-        p->fits = false;
-        cudaGetLastError();  // the next launch's error is its own
-    }
-    h->res_plans.push_back(own.release());
-    if (p->fits) *out = p;
+    if (e == cudaSuccess) return LPB_OK;
+    *ok = false;
+    cudaStreamSynchronize(h->stream);
+    if (p->mem) cudaFreeAsync(p->mem, h->stream);
+    p->mem = nullptr;
+    if (e != cudaErrorMemoryAllocation) return cuda_fail(e, "layout of the resident kernel");
+    p->fits = false;
+    p->lay.reset();
+    cudaGetLastError();  // the next launch's error is its own
     return LPB_OK;
 }
 
@@ -682,7 +729,15 @@ lpb_err res_choose(lpb_ctx* const* hs, Lane* const* lns, int count, ResShape* sh
         us_step += step_us<T>(p->pairs, longs, lns[i]->ncol) - fixed;
         fixed_us = std::max(fixed_us, fixed);
     }
-    if (smem > limit || us_res > 0.92 * (us_step + fixed_us)) return LPB_OK;
+    if (smem > limit || us_res > 0.92 * (us_step + fixed_us)) {
+        for (int i = 0; i < count; ++i) plans[i]->lay.reset();  // (measured again should another width want it)
+        return LPB_OK;
+    }
+    for (int i = 0; i < count; ++i) {
+        bool ok = false;
+        const lpb_err rc = res_ready<T>(hs[i], plans[i], kMostPairs, &ok);
+        if (rc != LPB_OK || !ok) return rc;
+    }
     shape->C = C;
     shape->threads = std::min(kResThreads, std::max(64, slices * 32));
     shape->smem = (size_t)smem;

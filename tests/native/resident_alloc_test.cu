@@ -1,7 +1,9 @@
 // Host-side check of the resident kernel's layouts (lpb_resident.cu) when the
 // device has no memory for them: the choice of the kernel is no error then, the
 // step kernels run, nothing of the layout is left behind and no second try
-// adds to it.  Runs on the stand-in runtime.  Prints "ok" or the first failure.
+// adds to it.  And of what making one costs the device's other users: nothing
+// waits for the whole device, and a batch that the step kernels run faster
+// allocates nothing.  Runs on the stand-in runtime.  Prints "ok" or the first failure.
 #include <cstdio>
 #include <vector>
 
@@ -42,6 +44,7 @@ int main() {
         ln.ncol = 16;
         ln.col_group.assign(ln.cap, 0);
         const size_t before = fake::live_bytes();
+        const long waits = fake::device_waits();
         for (int again = 0; again < 3; ++again) {
             ResShape shape;
             ResPlan* plan = nullptr;
@@ -55,6 +58,7 @@ int main() {
             if (done != (shape.C > 0)) return fail_at("the choice changes", k);
             if (h->res_plans.size() != 1) return fail_at("entries for one layout", (long)h->res_plans.size());
             if (!done && fake::live_bytes() != before) return fail_at("memory of a layout that is not used", k);
+            if (fake::device_waits() != waits) return fail_at("a wait for the whole device", fake::device_waits() - waits);
             if (fake::last_error()) return fail_at("an error is left for the next launch", k);
         }
         const long steps = fake::launches("k_step"), res = fake::launches("k_resident");
@@ -65,6 +69,20 @@ int main() {
         lpb_destroy(h);
         if (fake::live_bytes() != 0) return fail_at("memory left", k);
     }
+    // 30,000 entries in FP64: the step kernels' case
+    lpb_handle h = make(1000, 2000, 30, LPB_FP64);
+    if (!h) return fail_at("create", -1);
+    Lane& ln = h->lane[kPrecF64];
+    if (lane_reserve(h, ln, kPrecF64, 2, 1) != LPB_OK || ensure_check_ws(h, ln.cap) != LPB_OK) return fail_at("lane", -1);
+    ln.ncol = 2;
+    const size_t before = fake::live_bytes();
+    ResShape shape;
+    ResPlan* plan = nullptr;
+    Lane* lp = &ln;
+    if (res_choose<double>(&h, &lp, 1, &shape, &plan) != LPB_OK || shape.C != 0) return fail_at("the choice", shape.C);
+    if (fake::live_bytes() != before) return fail_at("memory of a layout that is not used", -1);
+    ln.ncol = 0;
+    lpb_destroy(h);
     std::printf("ok\n");
     return 0;
 }
