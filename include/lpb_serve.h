@@ -34,8 +34,11 @@ extern "C" {
 typedef struct lpb_server* lpb_server_t;
 
 typedef struct {
-    int64_t hbm_budget_bytes;  /* device bytes the server may hold for lanes and request buffers;
-                                  0 (default): 80% of the free device memory at create */
+    int64_t hbm_budget_bytes;  /* device bytes the server may hold for lanes, request buffers and the
+                                  layouts with which small matrices run whole intervals in one launch
+                                  (those give way to requests); what a handle holds when it is
+                                  attached is not counted.  0 (default): 80% of the free device
+                                  memory at create */
     int32_t lane_columns;      /* FP32 batch columns per attached matrix (default 256) */
     int32_t polish_columns;    /* polish-lane columns per attached matrix (default 64; 0: no polish lane) */
     int32_t max_groups;        /* concurrent requests per lane (default 64) */

@@ -18,6 +18,7 @@
 #pragma once
 
 #include <cstdint>
+#include <functional>
 #include <string>
 #include <vector>
 
@@ -153,6 +154,9 @@ struct lpb_ctx {
     // shape, and host copies of the row pointers of A~^T [0] and A~ [1]
     std::vector<lpb::ResPlan*> res_plans;
     std::vector<int> rp_host[2];
+    // a server's account of the layouts' device memory: asked before a layout
+    // takes bytes (false: the step kernels run), told when they go (negative)
+    std::function<bool(int64_t)> res_charge;
     lpb_lp_spec* specs_dev = nullptr;
     int specs_cap = 0;
     std::vector<void*> ws_allocs;
@@ -199,7 +203,9 @@ template <typename T>
 cudaError_t launch_resident(const IterPart<T>* parts, ResPlan* const* plans, int count, int L, const ResShape& shape,
                             cudaStream_t s);
 // Frees the handle's layouts; no launch that uses them may be in flight.
-void free_res_plans(lpb_ctx* h);
+// keep_stream: once the handle's stream has come to this point, without a wait
+// for the device; launches queued on that stream may use them.
+void free_res_plans(lpb_ctx* h, bool keep_stream = false);
 // first free run of count residual slots, or -1
 int lane_find_slots(const Lane& ln, int count);
 // a free group id, or -1

@@ -419,6 +419,7 @@ struct ResPlan {
     long long pairs = 0; // of a lane, both products
     std::unique_ptr<ResLayout[]> lay;  // until they are on the device
     void* mem = nullptr;               // both layouts and what they were filled from, one allocation
+    int64_t charged = 0;               // bytes of it on a server's account
     ResDir<double> dir[2];             // pointers; the value type follows prec
     // (rp: the row pointers of A~^T, then of A~); false: no such layouts
     bool measure(const std::vector<int>* rp, long long max_pairs) {
@@ -453,38 +454,51 @@ struct Carve {
     }
 };
 
+// where the arrays of a plan's two layouts lie in its allocation: those that
+// the host fills, then those that k_res_fill does
+struct ResPlaces {
+    struct {
+        size_t head, pword, lhead, np, flag, word, beg, len, pos, rec, va, ci;
+    } at[2];
+    size_t upload = 0, bytes = 0;
+};
+template <typename T>
+ResPlaces res_places(const ResPlan* plan) {
+    ResPlaces p;
+    Carve c;
+    for (int q = 0; q < 2; ++q) {
+        const ResLayout& l = plan->lay[q];
+        p.at[q].head = c.take(l.head.size() * sizeof(int2));
+        p.at[q].lhead = c.take(l.lhead.size() * sizeof(int4));
+        p.at[q].np = c.take(l.np.size() * 4);
+        p.at[q].flag = c.take(l.flag.size() * 4);
+        p.at[q].word = c.take(l.word.size() * 4);
+        p.at[q].pword = p.at[q].word + 4 * (size_t)l.places();  // the words of the piece slices are the last
+        p.at[q].beg = c.take(l.beg.size() * 4);
+        p.at[q].len = c.take(l.len.size() * 4);
+        p.at[q].pos = c.take(l.pos.size() * 4);
+    }
+    p.upload = c.bytes;
+    for (int q = 0; q < 2; ++q) {
+        const ResLayout& l = plan->lay[q];
+        p.at[q].rec = c.take((size_t)l.places() * sizeof(ResRec<T>));
+        p.at[q].va = c.take(32 * (size_t)l.total_pairs * sizeof(Pair<T>));
+        p.at[q].ci = c.take(32 * (size_t)l.total_pairs * 4);
+    }
+    p.bytes = c.bytes;
+    return p;
+}
+
 // The measured layouts on the device.  The allocation is stream-ordered and
 // the only wait is for the handle's own stream: cudaMalloc and cudaFree wait
 // for the whole device, and a server runs other matrices' intervals meanwhile.
 template <typename T>
-cudaError_t res_build(lpb_ctx* h, ResPlan* plan) {
+cudaError_t res_build(lpb_ctx* h, ResPlan* plan, const ResPlaces& places) {
     cudaStream_t s = h->stream;
     const IterData<T> it = lane_iter_data<T>(h, h->lane[0]);  // matrix and vectors only
     const Csr* csr[2] = {&h->At, &h->A};
-    struct Places {
-        size_t head, pword, lhead, np, flag, word, beg, len, pos, rec, va, ci;
-    } at[2];
-    Carve c;
-    for (int q = 0; q < 2; ++q) {
-        const ResLayout& l = plan->lay[q];
-        at[q].head = c.take(l.head.size() * sizeof(int2));
-        at[q].lhead = c.take(l.lhead.size() * sizeof(int4));
-        at[q].np = c.take(l.np.size() * 4);
-        at[q].flag = c.take(l.flag.size() * 4);
-        at[q].word = c.take(l.word.size() * 4);
-        at[q].pword = at[q].word + 4 * (size_t)l.places();  // the words of the piece slices are the last
-        at[q].beg = c.take(l.beg.size() * 4);
-        at[q].len = c.take(l.len.size() * 4);
-        at[q].pos = c.take(l.pos.size() * 4);
-    }
-    const size_t upload = c.bytes;
-    for (int q = 0; q < 2; ++q) {
-        const ResLayout& l = plan->lay[q];
-        at[q].rec = c.take((size_t)l.places() * sizeof(ResRec<T>));
-        at[q].va = c.take(32 * (size_t)l.total_pairs * sizeof(Pair<T>));
-        at[q].ci = c.take(32 * (size_t)l.total_pairs * 4);
-    }
-    std::vector<char> host(upload);
+    const auto& at = places.at;
+    std::vector<char> host(places.upload);
     auto put = [&](size_t to, const void* from, size_t bytes) {
         if (bytes) std::memcpy(host.data() + to, from, bytes);
     };
@@ -502,12 +516,12 @@ cudaError_t res_build(lpb_ctx* h, ResPlan* plan) {
         put(at[q].pos, l.pos.data(), l.pos.size() * 4);
     }
     cudaError_t e;
-    if ((e = cudaMallocAsync(&plan->mem, c.bytes, s)) != cudaSuccess) return e;
+    if ((e = cudaMallocAsync(&plan->mem, places.bytes, s)) != cudaSuccess) return e;
     char* mem = (char*)plan->mem;
-    if ((e = cudaMemcpyAsync(mem, host.data(), upload, cudaMemcpyHostToDevice, s)) != cudaSuccess) return e;
+    if ((e = cudaMemcpyAsync(mem, host.data(), places.upload, cudaMemcpyHostToDevice, s)) != cudaSuccess) return e;
     for (int q = 0; q < 2; ++q) {
         const ResLayout& l = plan->lay[q];
-        const Places& p = at[q];
+        const auto& p = at[q];
         ResDir<T> d{};
         d.shorts = l.shorts;
         d.longs = l.longs;
@@ -581,9 +595,11 @@ cudaError_t res_launch(const ResArgs<T>& g, int threads, size_t smem, cudaStream
 
 }  // namespace
 
-void free_res_plans(lpb_ctx* h) {
+void free_res_plans(lpb_ctx* h, bool keep_stream) {
+    if (!h->res_plans.empty()) h->ws_epoch += 1;  // captured intervals hold them
     for (ResPlan* p : h->res_plans) {
-        if (p->mem) cudaFree(p->mem);
+        if (p->mem) keep_stream ? cudaFreeAsync(p->mem, h->stream) : cudaFree(p->mem);
+        if (p->charged > 0 && h->res_charge) h->res_charge(-p->charged);
         delete p;
     }
     h->res_plans.clear();
@@ -657,18 +673,31 @@ lpb_err res_plan(lpb_ctx* h, int prec, int ncol, long long max_pairs, ResPlan** 
 }
 
 // A measured plan's layouts on the device, if they are not there yet; *ok =
-// false when no memory is left for them.  The step kernels need none and give
-// the same results, so that is no error of the solve.
+// false when no memory is left for them, or a server has none to give just
+// now.  The step kernels need none and give the same results, so that is no
+// error of the solve.
 template <typename T>
 lpb_err res_ready(lpb_ctx* h, ResPlan* p, long long max_pairs, bool* ok) {
     *ok = true;
     if (p->mem) return LPB_OK;
     cudaError_t e = cudaErrorMemoryAllocation;
     try {
-        if (p->lay || p->measure(h->rp_host, max_pairs)) e = res_build<T>(h, p);
+        if (p->lay || p->measure(h->rp_host, max_pairs)) {
+            const ResPlaces places = res_places<T>(p);
+            if (h->res_charge) {
+                if (!h->res_charge((int64_t)places.bytes)) {
+                    *ok = false;
+                    return LPB_OK;
+                }
+                p->charged = (int64_t)places.bytes;
+            }
+            e = res_build<T>(h, p, places);
+        }
     } catch (const std::bad_alloc&) {
     }
     if (e == cudaSuccess) return LPB_OK;
+    if (p->charged > 0) h->res_charge(-p->charged);
+    p->charged = 0;
     *ok = false;
     cudaStreamSynchronize(h->stream);
     if (p->mem) cudaFreeAsync(p->mem, h->stream);

@@ -61,6 +61,7 @@ struct Matrix {
     std::deque<Request*> pending;
     std::vector<Request*> running;
     int polish_prec = kPrecDfl;
+    bool wants_room = false;  // its next request fits in the budget once the layouts are given up
     bool in_flight = false;  // an interval is queued on the handle's stream
 };
 
@@ -86,11 +87,29 @@ struct lpb_server {
     std::vector<std::pair<int, void*>> to_free;
     int64_t next_id = 0;
     int64_t budget = 0, used = 0;
+    int64_t layouts = 0;  // of used: the resident kernel's layouts
     lpb_server_stats st{};
     double now() const { return std::chrono::duration<double>(Clock::now() - t0).count(); }
 };
 
 namespace {
+
+// some matrix's next request waits for the layouts' memory (srv->mu held)
+bool room_wanted(const lpb_server* srv) {
+    for (const auto& m : srv->mats)
+        if (m->wants_room) return true;
+    return false;
+}
+
+// lpb_ctx::res_charge of the attached handles: layouts take what requests
+// leave, and give it up when a request needs it (step_matrix)
+bool charge_layout(lpb_server* srv, int64_t bytes) {
+    std::lock_guard<std::mutex> lk(srv->mu);
+    if (bytes > 0 && (srv->used + bytes > srv->budget || room_wanted(srv))) return false;
+    srv->used += bytes;
+    srv->layouts += bytes;
+    return true;
+}
 
 int64_t lane_bytes(const lpb_ctx* h, int cols, int prec) {
     const int64_t ts = prec == kPrecF32 ? 4 : 8;
@@ -182,6 +201,7 @@ lpb_err admit_pending(lpb_server* srv, Matrix& M, bool& did_work) {
         int gid = -1, slot0 = -1;
         {
             std::lock_guard<std::mutex> lk(srv->mu);
+            M.wants_room = false;
             if (M.pending.empty()) return LPB_OK;
             r = M.pending.front();
             if (r->warm_request >= 0) {
@@ -201,7 +221,10 @@ lpb_err admit_pending(lpb_server* srv, Matrix& M, bool& did_work) {
             gid = lane_free_group(M.lane32, M.g32);
             slot0 = lane_find_slots(M.lane32, r->count);
             if (gid < 0 || slot0 < 0) return LPB_OK;
-            if (srv->used + r->footprint > srv->budget) return LPB_OK;
+            if (srv->used + r->footprint > srv->budget) {
+                M.wants_room = srv->used - srv->layouts + r->footprint <= srv->budget;
+                return LPB_OK;
+            }
             srv->used += r->footprint;
             r->charged = true;
             M.pending.pop_front();
@@ -349,6 +372,13 @@ lpb_err step_matrix(lpb_server* srv, Matrix& M, int mi, bool& did_work) {
         if ((rc = finish(srv, M, add, prof)) != LPB_OK) return rc;
         did_work = true;
     }
+    // (the last interval has ended, so no launch uses the layouts)
+    bool shed = false;
+    {
+        std::lock_guard<std::mutex> lk(srv->mu);
+        shed = room_wanted(srv);
+    }
+    if (shed) free_res_plans(M.h, true);
     if ((rc = admit_pending(srv, M, did_work)) != LPB_OK) return rc;
     if ((rc = launch(M, add, prof)) != LPB_OK) return rc;
     if (M.in_flight) {
@@ -484,6 +514,7 @@ lpb_err lpb_server_attach(lpb_server_t srv, lpb_handle h, int32_t* matrix_id) {
     }
     *matrix_id = (int32_t)srv->mats.size();
     Matrix* mp = M.get();
+    h->res_charge = [srv](int64_t bytes) { return charge_layout(srv, bytes); };
     srv->mats.push_back(std::move(M));
     srv->st.hbm_used_bytes = srv->used;
     srv->workers.emplace_back(worker_main, srv, mp, (int)*matrix_id);
@@ -674,6 +705,7 @@ void lpb_server_destroy(lpb_server_t srv) {
     cudaSetDevice(srv->device);
     for (auto& mp : srv->mats) {
         if (mp->h && mp->h->stream) cudaStreamSynchronize(mp->h->stream);
+        if (mp->h) mp->h->res_charge = nullptr;
         lane_free(mp->lane32);
         lane_free(mp->lanep);
     }

@@ -51,6 +51,8 @@ bool last_error() {
     Lock l(st().mu);
     return st().last != cudaSuccess;
 }
+std::function<void(void*, size_t)> on_read;
+
 long device_waits() {
     Lock l(st().mu);
     return st().waits;
@@ -131,8 +133,9 @@ cudaError_t cudaFreeHost(void* p) {
     std::free(p);
     return cudaSuccess;
 }
-cudaError_t cudaMemcpy(void* d, const void* s, size_t n, cudaMemcpyKind) {
+cudaError_t cudaMemcpy(void* d, const void* s, size_t n, cudaMemcpyKind k) {
     if (n) std::memcpy(d, s, n);
+    if (k == cudaMemcpyDeviceToHost && fake::on_read) fake::on_read(d, n);
     return cudaSuccess;
 }
 cudaError_t cudaMemcpyAsync(void* d, const void* s, size_t n, cudaMemcpyKind k, cudaStream_t) { return cudaMemcpy(d, s, n, k); }

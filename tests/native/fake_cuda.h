@@ -7,6 +7,7 @@
 #pragma once
 
 #include <cstddef>
+#include <functional>
 
 namespace fake {
 
@@ -21,5 +22,9 @@ long launches(const char* part);
 bool last_error();
 // calls so far that wait for the whole device: cudaMalloc and cudaFree
 long device_waits();
+
+// called after each copy from the device, with its destination and bytes (set
+// it while no other thread copies)
+extern std::function<void(void*, size_t)> on_read;
 
 }  // namespace fake

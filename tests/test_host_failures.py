@@ -1,4 +1,4 @@
-"""CPU: the library's host code when the device runs out of memory.  The
+"""CPU: the library's host code where device memory runs short.  The
 library's objects are linked with a stand-in for the CUDA runtime
 (tests/native/fake_cuda.cpp) that needs no GPU and fails allocations on demand."""
 import os
@@ -42,3 +42,7 @@ def test_a_threshold_change_without_memory_keeps_the_rows(objects, tmp_path):
 
 def test_a_layout_without_memory_leaves_the_step_kernels(objects, tmp_path):
     _run(objects, tmp_path, "resident_alloc_test")
+
+
+def test_a_servers_budget_covers_layouts_and_requests_come_first(objects, tmp_path):
+    _run(objects, tmp_path, "serve_layout_test")
