@@ -229,3 +229,28 @@ def test_steps_at_every_long_row_threshold(lpb, precision, thr, m, n, longest, l
         assert np.abs(y - ey[q]).max() <= tol * max(1.0, np.abs(ey[q] / dr).max()) * dr.max(), q
     b.free()
     h.close()
+
+
+def test_packed_rows_take_no_room_for_long_rows(lpb):
+    """A handle holds each entry once per orientation in the forms that the
+    checks and the long rows read (FP64, FP32, its low part, double-float, a
+    column: 28 bytes), and again only where it stands in a short row.  Here
+    all but 64 of eight million entries stand in rows and columns of 40 and
+    more: 56 bytes an entry, a generous 400 bytes a row or column, and 64 MB."""
+    import torch
+
+    m, n, dense = 72, 200_000, 40
+    lengths = np.array([n] * dense + [2] * (m - dense), dtype=np.int64)
+    ptr = np.concatenate([[0], np.cumsum(lengths)])
+    rng = np.random.default_rng(0)
+    cols = np.concatenate([np.tile(np.arange(n), dense), np.arange(2 * (m - dense))]).astype(np.int32)
+    lp = lpgen.LPData(m, n, ptr, cols, lpgen._signed_uniform(rng, cols.size), np.ones(n), np.full(m, -1.0), np.ones(m),
+                      np.zeros(n), np.ones(n), np.zeros(n), "dense_rows")
+    lpb.Handle(_lp(37, 50, 9, 1), precision=lpb.MIXED).close()  # the context and the library's own memory
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    h = lpb.Handle(lp, precision=lpb.MIXED, ruiz_iters=1, power_max_iter=2)
+    torch.cuda.synchronize()
+    held = before - torch.cuda.mem_get_info()[0]
+    h.close()
+    assert 56 * cols.size <= held <= 56 * cols.size + 400 * (m + n) + (64 << 20), held
