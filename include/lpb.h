@@ -78,7 +78,10 @@ typedef struct {
     uint64_t power_seed;            /* SplitMix64 seed of its start vector */
     double eps_infeas;              /* infeasibility tolerance; < 0 uses the solve's tol */
     int32_t detect_infeasibility;   /* 1: evaluate Eq. primal-infeas and dual-infeas */
-    int32_t profile;                /* 1: time every iteration kernel with CUDA events */
+    int32_t profile;                /* 1: time every iteration kernel with CUDA events.  A small
+                                       matrix, whose intervals otherwise run in one launch, runs
+                                       the step kernels then, with the same results; its solves
+                                       without profile are faster than these times say */
     void* cuda_stream;              /* cudaStream_t to run on, or NULL */
     int32_t device;                 /* CUDA device ordinal, or -1 for the current device */
     int32_t fp64_polish;            /* LPB_MIXED only: 1 (default) widens the remaining batch to
@@ -287,13 +290,17 @@ lpb_err lpb_set_tuning(lpb_handle h, const lpb_tuning* t);
 /* Autotuner: times the primal and dual steps on num_lps copies of the base
  * LP for every threshold in {8, 16, 32, 64, 128, 256} and shift in {0, ..., 4},
  * applies the fastest shape of each step to the handle and returns it in
- * *chosen (may be NULL).  Takes a few hundred step launches. */
+ * *chosen (may be NULL).  Takes a few hundred step launches.  It is the step
+ * kernels that are timed, also where solves of such a batch run whole
+ * intervals in one launch (small matrices), for which the shifts do not
+ * matter and the thresholds only say how long rows are cut. */
 lpb_err lpb_autotune(lpb_handle h, int32_t num_lps, lpb_tuning* chosen);
 
 /* Batch size by timing (Sec. 5: pick the N that maximises mat-vec products
- * per second): for each of count batch widths, the time of one iteration
- * (primal + dual step) on that many copies of the base LP, in microseconds,
- * into us_per_iter[i]; *best = the index with the most LP iterations per
+ * per second): for each of count batch widths, the time of one iteration on
+ * that many copies of the base LP, in microseconds, into us_per_iter[i]: the
+ * primal and the dual step, or, where a solve of that width runs whole
+ * intervals in one launch (small matrices), that launch's share; *best = the index with the most LP iterations per
  * second.  Widths must be in [1, 65536]. */
 lpb_err lpb_tune_batch(lpb_handle h, const int32_t* widths, int32_t count, double* us_per_iter, int32_t* best);
 

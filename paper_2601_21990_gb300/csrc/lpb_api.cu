@@ -361,11 +361,14 @@ lpb_err solve_joint_impl(const std::vector<lpb_ctx*>& hs, const int32_t* num_lps
     return rc;
 }
 
-// Times R plain iterations (no check) of `count` copies of the base LP on the
-// handle's lane of its precision: per-iteration microseconds of the primal and
-// dual steps (medians over the iterations).
+// Times plain iterations (no check) of `count` copies of the base LP on the
+// handle's lane of its precision, in microseconds an iteration: the primal and
+// dual steps (medians over R of them) into *us_primal and *us_dual; or, where
+// us_resident is given and a solve of that batch runs whole intervals in one
+// launch, that kernel (the median of its launches) into *us_resident, which
+// is negative otherwise.
 template <typename T>
-lpb_err time_steps(lpb_ctx* h, int count, int R, double* us_primal, double* us_dual) {
+lpb_err time_steps(lpb_ctx* h, int count, int R, double* us_primal, double* us_dual, double* us_resident) {
     lpb_err rc;
     cudaStream_t s = h->stream;
     Lane& ln = h->lane[prec_of<T>()];
@@ -397,7 +400,29 @@ lpb_err time_steps(lpb_ctx* h, int count, int R, double* us_primal, double* us_d
     for (auto& e : ev) CU(cudaEventCreate(&e));
     std::vector<float> tp, td;
     cudaError_t ce = cudaSuccess;
-    for (int t = 0; t < R + 2 && ce == cudaSuccess; ++t) {
+    ResShape shape;
+    ResPlan* plan = nullptr;
+    Lane* lp = &ln;
+    if (us_resident) *us_resident = -1.0;
+    // (a solve that times its steps, profile = 1, runs the step kernels)
+    if (us_resident && !h->opt.profile) rc = res_choose<T>(&h, &lp, 1, &shape, &plan);
+    if (rc == LPB_OK && shape.C > 0) {
+        const IterPart<T> q{id, ib, ln.cap, ln.ncol, h->opt.check_every, 0, hal};
+        const int L = std::min(h->opt.check_every, 64);
+        for (int t = 0; t < 7 && ce == cudaSuccess; ++t) {
+            ce = cudaEventRecord(ev[0], s);
+            if (ce == cudaSuccess) ce = launch_resident<T>(&q, &plan, 1, L, shape, s);
+            if (ce == cudaSuccess) ce = cudaEventRecord(ev[1], s);
+            if (ce == cudaSuccess) ce = cudaStreamSynchronize(s);
+            float a = 0.f;
+            if (ce == cudaSuccess && t >= 2) {
+                cudaEventElapsedTime(&a, ev[0], ev[1]);
+                tp.push_back(a / (float)L);
+            }
+        }
+        td.push_back(0.f);
+    }
+    for (int t = 0; rc == LPB_OK && shape.C == 0 && t < R + 2 && ce == cudaSuccess; ++t) {
         ce = launch_iteration<T>(id, ib, ln.cap, ln.ncol, hal, t % h->opt.check_every, h->opt.check_every, 0, false,
                                  false, s, ev);
         if (ce == cudaSuccess) ce = cudaStreamSynchronize(s);
@@ -416,19 +441,21 @@ lpb_err time_steps(lpb_ctx* h, int count, int R, double* us_primal, double* us_d
     std::fill(ln.col_group.begin(), ln.col_group.end(), -1);
     cudaMemsetAsync(ln.ctl, 0, sizeof(Control) * ln.gcap, s);
     cudaStreamSynchronize(s);
+    if (rc != LPB_OK) return rc;
     if (ce != cudaSuccess) return cuda_fail(ce, "timed steps");
     std::sort(tp.begin(), tp.end());
     std::sort(td.begin(), td.end());
+    if (shape.C > 0) *us_resident = 1e3 * tp[tp.size() / 2];
     *us_primal = 1e3 * tp[tp.size() / 2];
     *us_dual = 1e3 * td[td.size() / 2];
     return LPB_OK;
 }
 
-lpb_err time_steps_any(lpb_ctx* h, int count, int R, double* up, double* ud) {
+lpb_err time_steps_any(lpb_ctx* h, int count, int R, double* up, double* ud, double* ures) {
     const lpb_err rc = rows_ready(h);
     if (rc != LPB_OK) return rc;
-    return h->opt.precision == LPB_MIXED ? time_steps<float>(h, count, R, up, ud)
-                                         : time_steps<double>(h, count, R, up, ud);
+    return h->opt.precision == LPB_MIXED ? time_steps<float>(h, count, R, up, ud, ures)
+                                         : time_steps<double>(h, count, R, up, ud, ures);
 }
 
 // the packed short rows of A~ or A~^T in the iterate types that the handle's
@@ -979,7 +1006,7 @@ lpb_err lpb_autotune(lpb_handle h, int32_t num_lps, lpb_tuning* chosen) {
             if ((rc = apply_shape(h, h->At, thr, sh)) != LPB_OK) return rc;
             if ((rc = apply_shape(h, h->A, thr, sh)) != LPB_OK) return rc;
             double up = 0.0, ud = 0.0;
-            if ((rc = time_steps_any(h, num_lps, 9, &up, &ud)) != LPB_OK) return rc;
+            if ((rc = time_steps_any(h, num_lps, 9, &up, &ud, nullptr)) != LPB_OK) return rc;
             if (up < best_p) {
                 best_p = up;
                 bp_thr = thr;
@@ -1005,11 +1032,11 @@ lpb_err lpb_tune_batch(lpb_handle h, const int32_t* widths, int32_t count, doubl
     DeviceGuard guard(h->device);
     double best_rate = -1.0;
     for (int32_t i = 0; i < count; ++i) {
-        double up = 0.0, ud = 0.0;
-        lpb_err rc = time_steps_any(h, widths[i], 9, &up, &ud);
+        double up = 0.0, ud = 0.0, ures = -1.0;
+        lpb_err rc = time_steps_any(h, widths[i], 9, &up, &ud, &ures);
         if (rc != LPB_OK) return rc;
-        us_per_iter[i] = up + ud;
-        const double rate = widths[i] / (up + ud);
+        us_per_iter[i] = ures >= 0.0 ? ures : up + ud;
+        const double rate = widths[i] / us_per_iter[i];
         if (rate > best_rate) {
             best_rate = rate;
             if (best) *best = i;

@@ -254,3 +254,25 @@ def test_packed_rows_take_no_room_for_long_rows(lpb):
     held = before - torch.cuda.mem_get_info()[0]
     h.close()
     assert 56 * cols.size <= held <= 56 * cols.size + 400 * (m + n) + (64 << 20), held
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+def test_tune_batch_times_the_kernel_that_a_solve_runs(lpb, precision):
+    """On a small matrix a solve runs whole intervals in one launch, in well
+    under the time of its steps one by one: lpb_tune_batch reports that kernel,
+    and the step kernels on a handle whose solves time them (profile = 1)."""
+    lp = _lp(200, 400, 20, 7)
+    opts = dict(precision=lpb.FP64 if precision == "fp64" else lpb.MIXED)
+    us = {}
+    for profile in (0, 1):
+        h = lpb.Handle(lp, profile=profile, **opts)
+        sp = _specs(lp, 16, 0)
+        b = h.solve(lpb.specs_array(sp.kind, sp.var, sp.lo, sp.hi, sp.sign), tol=1e-12, max_iter=128)
+        p = b.profile()
+        assert (p.kernels < sum(p.launches[:2])) == (profile == 0)
+        us[profile] = h.tune_batch([16])[0][0]
+        if profile:
+            steps = 1e3 * (p.ms[0] + p.ms[1]) / p.launches[0]
+        b.free()
+        h.close()
+    assert us[0] < 0.85 * us[1] and us[0] < 0.85 * steps, (us, steps)
