@@ -69,7 +69,7 @@ struct ResDir {
 
 template <typename T>
 struct ResPart {
-    int ld, ncol, ce, uni, slots;
+    int ld, ncol, ce, uni;
     T *Xbar, *Y, *Xh, *DX, *Yh, *DY, *DYp;
     const T *X0, *Y0;
     const T* hal;
@@ -800,7 +800,6 @@ cudaError_t launch_resident(const IterPart<T>* parts, ResPlan* const* plans, int
         a.Y0 = q.b.Y0;
         a.hal = q.hal;
         a.col = q.d.col;
-        a.slots = plans[i]->slots;
         a.p = typed<T>(plans[i]->dir[0]);
         a.d = typed<T>(plans[i]->dir[1]);
     }

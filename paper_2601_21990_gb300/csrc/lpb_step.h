@@ -57,7 +57,7 @@ constexpr int kFlat = 4;
 constexpr int kNarrowLanes = 2;
 
 template <typename T, int G, int B> struct MinBlocks {
-    static constexpr int v = B > kFlat                       ? (B > 8 ? 3 : LPB_STEP_MIN_BLOCKS_DEEP)
+    static constexpr int v = B > kFlat                       ? LPB_STEP_MIN_BLOCKS_DEEP
                              : std::is_same<T, double>::value ? LPB_STEP_MIN_BLOCKS_F64
                              : std::is_same<T, dfloat>::value ? LPB_STEP_MIN_BLOCKS_DF
                              : G >= 32                        ? LPB_STEP_MIN_BLOCKS_WIDE
@@ -307,11 +307,8 @@ template <typename T>
 struct StepArgs {
     // sparse operator (rows of A~^T for the primal step, of A~ for the dual step)
     int rows;
-    const int* rp;
     const int* ci;
     const T* va;
-    const int* long_rows;
-    int n_long;
     // the other rows in the order in which they are taken, their entries in
     // fours, their cost and bounds (Csr::srec ..)
     const int4* srec;
@@ -456,7 +453,7 @@ struct RowK {
     T c, lo, hi;
 };
 
-// the same by plain loads (long rows)
+// the point and its anchor, by plain loads (previous kernels write them)
 template <typename T, int V, bool PRIMAL>
 __device__ __forceinline__ RowOwn<T, V> load_own(const StepArgs<T>& a, int row, int col0) {
     RowOwn<T, V> o;
@@ -883,11 +880,8 @@ StepArgs<T> step_args(bool primal, const IterData<T>& d, const IterBufs<T>& b, i
     const Csr& c = primal ? d.At : d.A;
     StepArgs<T> a{};
     a.rows = c.rows;
-    a.rp = c.rp;
     a.ci = c.ci;
     a.va = primal ? d.at_vals : d.a_vals;
-    a.long_rows = c.long_rows;
-    a.n_long = c.n_long;
     a.srec = row_group_lanes<T>(ncol, c.g_shift) <= kNarrowLanes ? c.nrec : c.srec;
     a.pci = c.pci;
     a.pva = primal ? d.at_pv : d.a_pv;
