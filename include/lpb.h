@@ -199,12 +199,14 @@ enum { LPB_MAX_JOINT = 64 };
  * (as lpb_solve, no warm start).  Every iteration runs the primal steps of
  * all batches still iterating as one kernel launch, then their dual steps
  * as one launch (one launch per row-group width among the batches and per
- * 8 batches), and each batch's check after the interval, all on the first
- * handle's stream; with the first handle's use_graphs each interval is one
- * CUDA graph.  A batch that finishes leaves the joint launches; one that
- * stalls at FP32 resolution (LPB_MIXED with fp64_polish) leaves them and is
- * polished on its own handle and stream.  Each result is bitwise the one
- * lpb_solve gives for that batch alone.  Event timing (profile = 1) is not
+ * 8 batches; where all matrices are small, whole intervals in one launch), on
+ * the first handle's stream; then the batches' checks, side by side on their
+ * handles' streams (on the first handle's where the caller gave the stream);
+ * with the first handle's use_graphs each interval is one CUDA graph.  A batch that finishes leaves the joint launches; one that
+ * stalls at FP32 resolution (LPB_MIXED with fp64_polish) leaves them, and
+ * when all have finished or stalled, the stalled ones polish together on their
+ * handles' polish lanes.  Each result is bitwise the one lpb_solve gives for
+ * that batch alone (while its points are finite).  Event timing (profile = 1) is not
  * taken; each batch's lpb_profile counts its share of the launches as if
  * solved alone.
  * Rejects (LPB_ERR_INVALID_ARG): count outside [1, LPB_MAX_JOINT], a NULL
@@ -284,7 +286,11 @@ typedef struct {
 } lpb_tuning;
 
 lpb_err lpb_get_tuning(lpb_handle h, lpb_tuning* t);
-/* thresholds >= 1, shifts in [0, 5]; LPB_ERR_INVALID_ARG otherwise */
+/* thresholds >= 1 (2^31 - 1: no row is cut), shifts in [0, 5];
+ * LPB_ERR_INVALID_ARG otherwise.  A change of a threshold lays the rows out
+ * anew; when that runs out of memory (LPB_ERR_OOM), the old threshold of that
+ * matrix stays, and where not even its rows can be laid out again, solves
+ * return LPB_ERR_OOM until a later change succeeds. */
 lpb_err lpb_set_tuning(lpb_handle h, const lpb_tuning* t);
 
 /* Autotuner: times the primal and dual steps on num_lps copies of the base

@@ -12,8 +12,11 @@
 //
 // Every row is summed in the order in which the step kernel at this batch
 // width sums it (pieces and segments of long rows among it) and the
-// elementwise steps are the same code (primal_element, dual_element): the
-// iterates are bitwise those of the step kernels.
+// elementwise steps are the same code (primal_element, dual_element): while
+// the points are finite, the iterates are bitwise those of the step kernels.
+// (A lane that is shorter than its slice adds 0 times its first entry's point,
+// a packed row of an odd length 0 times its last one's: an infinite point
+// can make the one sum NaN and leave the other infinite.)
 //
 // Why one block and no cluster: splitting the rows over the blocks of a
 // cluster needs each block's rows in every other block's shared memory twice
@@ -609,9 +612,9 @@ namespace {
 
 // Estimated microseconds of an iteration: of the resident kernel for a layout
 // of `pairs` (of a lane, both products) and C columns a block, and of the step
-// kernels for the same matrix at ncol columns.  Fitted on GB300 over matrices
-// of 200 to 2750 rows and 1 to 900 LPs; the constants are where each bound
-// lies:
+// kernels for the same matrix at ncol columns.  Fitted on GB300 at 2070 MHz
+// over matrices of 200 to 2750 rows and 1 to 900 LPs; the constants are where
+// each bound lies:
 //   resident, FP32: a pair of entries per lane takes the block 7 ns (issue,
 //   bank conflicts of the gathers), 14 ns once the entries exceed what L1
 //   holds beside the resident blocks (550 pairs, 210 KB); FP64 and

@@ -1,7 +1,11 @@
 // lpb_resident.h -- the layout of a matrix for the resident interval kernel
 // (lpb_resident.cu): which thread takes a row, and the order in which a
 // row's entries are summed.  Plain host code, checked without a GPU by
-// tests/native/resident_layout_test.cu.
+// tests/native/resident_layout_test.cu.  Rows sorted by length and taken in
+// slices of as many rows as lanes, each padded to its longest, are the
+// SELL-C-sigma format of Kreutzer, Hager, Wellein, Fehske and Bishop (SIAM J.
+// Sci. Comput. 36(5), 2014), here with one window over all rows; cutting the
+// long rows in the step kernels' pieces is this kernel's own.
 #pragma once
 
 #include <algorithm>

@@ -226,9 +226,11 @@ __global__ void k_long_scatter(const int* __restrict__ flag, const int* __restri
 // ---------------------------------------------------------------------------
 // short rows in the order of the step kernels
 // ---------------------------------------------------------------------------
-// Windows of kWindow rows, each sorted by length, longest first: the row
-// groups of a warp then take rows of about the same length, and rows that lie
-// near one another stay near (a window's rows share what they gather in L2).
+// Windows of kWindow rows, each sorted by length, longest first (the windows
+// of the SELL-C-sigma format of Kreutzer, Hager, Wellein, Fehske and Bishop,
+// SIAM J. Sci. Comput. 36(5), 2014): the row groups of a warp then take rows
+// of about the same length, and rows that lie near one another stay near (a
+// window's rows share what they gather in L2).
 // Row groups of one or two lanes take the rows from a second list, of windows
 // of kNarrow rows, which a block or two takes at once: their points' sixteen or
 // 32 bytes a row are whole lines only together (256 iterations of 2 LPs on
