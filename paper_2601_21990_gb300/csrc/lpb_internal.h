@@ -75,11 +75,11 @@ struct Csr {
     float* v32lo = nullptr;     // v64 - v32 rounded to FP32: (v32, v32lo) is v64 in double-float
     int* long_rows = nullptr;   // rows with > long_thr entries
     int n_long = 0;
-    // The other rows as the step kernels take them (build_short_rows): in
-    // windows sorted by length, each row's entries together, from a multiple of
-    // four on, and its cost and bounds beside its record.
-    int4* nrec = nullptr;       // the same rows for one or two lanes a row: row, fours, pairs, place in srec
-    int4* srec = nullptr;       // row, its first four entries (entry index / 4), pairs of entries, entries
+    // The other rows as the step kernels take them (build_short_rows): each
+    // row's entries together, from a multiple of four on, in windows of rows
+    // sorted by length, and its cost and bounds at its record's place.
+    int4* srec = nullptr;       // in that order: row, its first four entries (entry index / 4), pairs, place
+    int4* nrec = nullptr;       // the same records in the rows' own order
     int n_short = 0;
     int* pci = nullptr;         // entries: columns, and values in the iterate types in use
     float* pv32 = nullptr;

@@ -226,20 +226,17 @@ __global__ void k_long_scatter(const int* __restrict__ flag, const int* __restri
 // ---------------------------------------------------------------------------
 // short rows in the order of the step kernels
 // ---------------------------------------------------------------------------
-// Windows of kWindow rows, each sorted by length, longest first (the windows
-// of the SELL-C-sigma format of Kreutzer, Hager, Wellein, Fehske and Bishop,
-// SIAM J. Sci. Comput. 36(5), 2014): the row groups of a warp then take rows
-// of about the same length, and rows that lie near one another stay near (a
-// window's rows share what they gather in L2).
-// Row groups of one or two lanes take the rows from a second list, of windows
-// of kNarrow rows, which a block or two takes at once: their points' sixteen or
-// 32 bytes a row are whole lines only together (256 iterations of 2 LPs on
-// 200k x 400k: 19.6 ms in the one order, 17.5 in the other; of 2 LPs on 20k x
-// 50k: 4.3 and 3.8; 16 columns and more lose up to 13% by the shorter windows).
-constexpr int kWindow = 2048, kNarrow = 128;
+// Two lists (Csr::srec, Csr::nrec; step_args says which step takes which).
+// The first: windows of kWindow rows, each sorted by length, longest first (the
+// windows of the SELL-C-sigma format of Kreutzer, Hager, Wellein, Fehske and
+// Bishop, SIAM J. Sci. Comput. 36(5), 2014): the row groups of a warp then take
+// rows of about the same length, and rows that lie near one another stay near
+// (a window's rows share what they gather in L2).  The second: the rows as they
+// stand, so that a warp's narrow row groups read and write their points, 16 to
+// 128 bytes a row, in whole lines.
+constexpr int kWindow = 2048;
 
 // per window: its rows of at most thr entries
-template <int kWindow>
 __global__ void __launch_bounds__(256) k_short_count(const int* __restrict__ rp, int rows, int thr,
                                                      int* __restrict__ cnt) {
     __shared__ int sum;
@@ -258,7 +255,6 @@ __global__ void __launch_bounds__(256) k_short_count(const int* __restrict__ rp,
 // one block per window: bitonic sort of the places' keys (short_key), the
 // rows of more than thr entries and the places past the last row at the end;
 // equal lengths keep their order
-template <int kWindow>
 __global__ void __launch_bounds__(1024) k_short_order(const int* __restrict__ rp, int rows, int thr,
                                                       const int* __restrict__ first, int4* __restrict__ out) {
     __shared__ unsigned long long key[kWindow];
@@ -301,18 +297,28 @@ __global__ void k_short_place(int4* __restrict__ rec, int n, const int* __restri
     }
 }
 
-// the record of each row, and the narrow list's records from it: their last
-// word is that record's place, where the row's cost and bounds stand
+// the record of each row, and from it the records in the rows' order (first:
+// how many short rows stand before a row)
 __global__ void k_short_where(const int4* __restrict__ rec, int n, int* __restrict__ place) {
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) place[rec[i].x] = i;
 }
-__global__ void k_short_narrow(const int4* __restrict__ rec, const int* __restrict__ place, int n,
+__global__ void k_short_flags(const int* __restrict__ rp, int rows, int thr, int* __restrict__ flag) {
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < rows; i += gridDim.x * blockDim.x)
+        flag[i] = rp[i + 1] - rp[i] <= thr ? 1 : 0;
+}
+__global__ void k_short_narrow(const int4* __restrict__ rec, const int* __restrict__ place,
+                               const int* __restrict__ rp, int rows, int thr, const int* __restrict__ first,
                                int4* __restrict__ out) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        const int p = place[out[i].x];
-        const int4 r = rec[p];
-        out[i] = make_int4(r.x, r.y, r.z, p);
-    }
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < rows; i += gridDim.x * blockDim.x)
+        if (rp[i + 1] - rp[i] <= thr) {
+            const int p = place[i];
+            const int4 r = rec[p];
+            out[first[i]] = make_int4(i, r.y, r.z, p);
+        }
+}
+// (last: the entries are counted by the word until then)
+__global__ void k_short_self(int4* __restrict__ rec, int n) {
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) rec[i].w = i;
 }
 
 // columns of the packed entries, and their values and the rows' vectors: a
@@ -892,20 +898,15 @@ cudaError_t build_short_rows(Csr& a, RowVectors<float> v32, RowVectors<double> v
     if (v32.vals) a.pk32 = (float*)(mem + at_k32);
     if (v64.vals) a.pk64 = (double*)(mem + at_k64);
     if (vdf.vals) a.pkdf = (dfloat*)(mem + at_kdf);
-    const int windows = (a.rows + kWindow - 1) / kWindow, narrow = (a.rows + kNarrow - 1) / kNarrow;
+    const int windows = (a.rows + kWindow - 1) / kWindow;
     const size_t most = std::max((size_t)a.rows, (size_t)n);
     StreamMem scratch(s);
     if ((e = scratch.take(sizeof(int) * (most * 2 + 1))) != cudaSuccess) return e;
     int *cnt = (int*)scratch.p, *first = cnt + most, *total = first + most;
-    k_short_count<kNarrow><<<narrow, kNarrow, 0, s>>>(a.rp, a.rows, a.long_thr, cnt);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    if ((e = exclusive_scan_i32(cnt, first, narrow, nullptr, s)) != cudaSuccess) return e;
-    k_short_order<kNarrow><<<narrow, kNarrow, 0, s>>>(a.rp, a.rows, a.long_thr, first, a.nrec);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    k_short_count<kWindow><<<windows, 256, 0, s>>>(a.rp, a.rows, a.long_thr, cnt);
+    k_short_count<<<windows, 256, 0, s>>>(a.rp, a.rows, a.long_thr, cnt);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if ((e = exclusive_scan_i32(cnt, first, windows, nullptr, s)) != cudaSuccess) return e;
-    k_short_order<kWindow><<<windows, 1024, 0, s>>>(a.rp, a.rows, a.long_thr, first, a.srec);
+    k_short_order<<<windows, 1024, 0, s>>>(a.rp, a.rows, a.long_thr, first, a.srec);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     k_short_fours<<<grid_for(n, 256), 256, 0, s>>>(a.srec, n, cnt);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
@@ -914,9 +915,12 @@ cudaError_t build_short_rows(Csr& a, RowVectors<float> v32, RowVectors<double> v
     if ((e = cudaMemcpyAsync(&fours, total, sizeof(int), cudaMemcpyDeviceToHost, s)) != cudaSuccess) return e;
     k_short_place<<<grid_for(n, 256), 256, 0, s>>>(a.srec, n, first);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    k_short_flags<<<grid_for(a.rows, 256), 256, 0, s>>>(a.rp, a.rows, a.long_thr, cnt);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if ((e = exclusive_scan_i32(cnt, first, a.rows, nullptr, s)) != cudaSuccess) return e;
     k_short_where<<<grid_for(n, 256), 256, 0, s>>>(a.srec, n, cnt);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    k_short_narrow<<<grid_for(n, 256), 256, 0, s>>>(a.srec, cnt, n, a.nrec);
+    k_short_narrow<<<grid_for(a.rows, 256), 256, 0, s>>>(a.srec, cnt, a.rp, a.rows, a.long_thr, first, a.nrec);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     // the entries: as many as the short rows have, the long rows' stay where they are
     if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return e;
@@ -935,6 +939,8 @@ cudaError_t build_short_rows(Csr& a, RowVectors<float> v32, RowVectors<double> v
     if ((e = pack_vals<float>(a, n, v32, a.pv32, a.pk32, s)) != cudaSuccess) return e;
     if ((e = pack_vals<double>(a, n, v64, a.pv64, a.pk64, s)) != cudaSuccess) return e;
     if ((e = pack_vals<dfloat>(a, n, vdf, a.pvdf, a.pkdf, s)) != cudaSuccess) return e;
+    k_short_self<<<grid_for(n, 256), 256, 0, s>>>(a.srec, n);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
     a.n_short = n;
     return cudaSuccess;
 }

@@ -53,9 +53,6 @@ template <> struct Vec<dfloat> { static constexpr int V = 2; };
 template <int G> constexpr int kDeep = G >= 32 ? 0 : 8;
 constexpr int kFlat = 4;
 
-// Row groups of at most so many lanes take the short rows from Csr::nrec.
-constexpr int kNarrowLanes = 2;
-
 template <typename T, int G, int B> struct MinBlocks {
     static constexpr int v = B > kFlat                       ? LPB_STEP_MIN_BLOCKS_DEEP
                              : std::is_same<T, double>::value ? LPB_STEP_MIN_BLOCKS_F64
@@ -363,8 +360,8 @@ __device__ __forceinline__ bool long_row_reduce(T (&acc)[V], T* red) {
 // they are so many that a block each would be more than a wave of mostly
 // prologue (long_per): 4 for one lane, 2 for two.  Measured with a block a
 // segment and with these: 2 LPs on the 20k x 50k power-law matrix (1500
-// segments) 5.0 and 4.4 ms a pass of 256 iterations (3.7 with the rows in the
-// narrow order), 8 LPs 4.1 and 3.7; on 100k x 200k with 50 long rows (200
+// segments) 5.0 and 4.4 ms a pass of 256 iterations (3.5 with the short rows
+// in their own order), 8 LPs 4.1 and 3.7; on 100k x 200k with 50 long rows (200
 // segments), 2 LPs, 6.05 and 6.4.
 template <int G> constexpr int kSegPer = G <= 2 ? 4 / G : 1;
 template <int G>
@@ -766,7 +763,7 @@ __device__ __forceinline__ void step_body(const StepArgs<T>& a, const int bx, co
     pdl_wait(a.pdl);
 #pragma unroll 1
     for (; i < a.n_short; i += stride) {
-        const int row = rec.x, first = rec.y, pairs = rec.z, place = G <= kNarrowLanes ? rec.w : i;
+        const int row = rec.x, first = rec.y, pairs = rec.z, place = rec.w;
         if (i + stride < a.n_short) rec = __ldg(a.srec + i + stride);
         T acc[V];
 #pragma unroll
@@ -870,6 +867,26 @@ inline cudaError_t l2_bytes(long long* out) {
     return cudaSuccess;
 }
 
+// Whether a step takes the short rows in their own order (Csr::nrec) and not
+// by length (Csr::srec); own: the bytes of the rows' two own blocks.  By
+// length, a warp's row groups run about as many entries each, but the rows'
+// points lie apart.  Narrow row groups' points (16 bytes a lane) then come in
+// parts of lines, the more so from HBM, where the primal step, of few entries a
+// row, moves more of its own points than it gathers.  FP64, bound by its pipe,
+// wants the equal lengths at every width; double-float lies between.
+// Microseconds of a step kernel pair by length and in the rows' order: FP32,
+// 4 LPs on 200k x 400k 63 and 60, 8 LPs on 1M x 2M 245 and 220, 16 LPs 474 and
+// 390, 32 LPs 656 and 600 (with 32 LPs on 100k x 100k 40 and 44, and on 200k x
+// 400k the dual step 78 and 90: by length); double-float, 2 LPs on 400k x 1M
+// 134 and 120, 4 LPs 122 and 128, 8 LPs 206 and 195, on 1M x 2M 512 and 454, on
+// 200k x 400k 110 and 114; FP64, 8 LPs on 200k x 400k 311 and 345.
+template <typename T>
+bool natural_order(int lanes, bool primal, long long own, long long l2) {
+    if (std::is_same<T, double>::value) return false;
+    const int any = std::is_same<T, float>::value ? 4 : 1, far = std::is_same<T, float>::value ? 8 : 4;
+    return lanes <= any || (lanes <= far && primal && 2 * own > l2);
+}
+
 // The arguments of one matrix's primal step (rows of A~^T gathering Y) or
 // dual step (rows of A~ gathering Xbar) at iteration t of its interval;
 // pdl is left to the caller.  l2: the device's L2 bytes, which decide whether
@@ -882,7 +899,9 @@ StepArgs<T> step_args(bool primal, const IterData<T>& d, const IterBufs<T>& b, i
     a.rows = c.rows;
     a.ci = c.ci;
     a.va = primal ? d.at_vals : d.a_vals;
-    a.srec = row_group_lanes<T>(ncol, c.g_shift) <= kNarrowLanes ? c.nrec : c.srec;
+    const int lanes = row_group_lanes<T>(ncol, c.g_shift);
+    const long long own = 2LL * c.rows * ld * (long long)sizeof(T);
+    a.srec = natural_order<T>(lanes, primal, own, l2) ? c.nrec : c.srec;
     a.pci = c.pci;
     a.pva = primal ? d.at_pv : d.a_pv;
     a.pk = primal ? d.at_pk : d.a_pk;

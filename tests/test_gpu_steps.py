@@ -276,3 +276,32 @@ def test_tune_batch_times_the_kernel_that_a_solve_runs(lpb, precision):
         b.free()
         h.close()
     assert us[0] < 0.85 * us[1] and us[0] < 0.85 * steps, (us, steps)
+
+
+@pytest.mark.parametrize("lps,lanes", [(3, 1), (7, 2), (13, 4), (30, 8)])
+def test_row_orders_agree_on_a_large_matrix(lpb, lps, lanes):
+    """Narrow batches take the rows as they stand, wider ones by length, and at
+    eight lanes the primal step of a matrix whose points exceed L2 the former:
+    bit for bit the same points and results, as a short row is summed in its
+    own order whoever takes it.  64 LPs (16 lanes, by length) against the first
+    of them alone; one check, so no restart couples them."""
+    m, n = 150_000, 600_000
+    rng = np.random.default_rng(1)
+    lengths = rng.integers(0, 9, m)
+    ptr = np.concatenate([[0], np.cumsum(lengths)]).astype(np.int64)
+    cols = np.concatenate([np.sort(c) for c in np.split(rng.integers(0, n, ptr[-1]), ptr[1:-1])]).astype(np.int32)
+    x0 = rng.uniform(0.0, 10.0, n)
+    lp = lpgen.LPData(m, n, ptr, cols, lpgen._signed_uniform(rng, cols.size), rng.standard_normal(n), None, None,
+                      np.zeros(n), np.full(n, 10.0), x0, "orders")
+    lpgen._rows_around(lp, x0, rng)
+    sp = _specs(lp, 64, 3)
+    specs = lpb.specs_array(sp.kind, sp.var, sp.lo, sp.hi, sp.sign)
+    h = lpb.Handle(lp, precision=lpb.MIXED, power_max_iter=50)
+    wide = h.solve(specs, tol=1e-12, max_iter=64)
+    narrow = h.solve(specs[:lps], tol=1e-12, max_iter=64)
+    assert np.array_equal(wide.results()[:lps], narrow.results())
+    for q in (0, lps // 2, lps - 1):
+        for a, b in zip(wide.result(q)[1:], narrow.result(q)[1:]):
+            assert np.array_equal(a, b), q
+    wide.free(), narrow.free()
+    h.close()
