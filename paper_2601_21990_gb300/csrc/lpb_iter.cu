@@ -49,9 +49,9 @@ cudaError_t launch_k(StepArgs<T> a, bool if_fits, bool* fits, cudaStream_t s) {
     constexpr int V = Vec<T>::V, GPB = kBlock / G, TN = G * V;
     static std::atomic<int> shape[kShapeDevices];  // static storage: starts at 0
     int sms = 0, per_sm = 0;
-    const cudaError_t e = launch_shape(shape, k_step<T, G, B, CHECK, PRIMAL>, long_smem<T, G>(1, kSegPer<G>), &sms, &per_sm);
+    const cudaError_t e = launch_shape(shape, k_step<T, G, B, CHECK, PRIMAL>, long_smem<T, G>(1, kSegPer<T, G>), &sms, &per_sm);
     if (e != cudaSuccess) return e;
-    a.per = long_per<G>(a.n_lseg, sms);
+    a.per = long_per<T, G>(a.n_lseg, sms);
     const int nlb = (a.n_lseg + a.per - 1) / a.per, need = (a.n_short + GPB - 1) / GPB, tiles = (a.ncol + TN - 1) / TN;
     *fits = ((long long)nlb + need) * tiles <= (long long)sms * per_sm;
     if (if_fits && !*fits) return cudaSuccess;

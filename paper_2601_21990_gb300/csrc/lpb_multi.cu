@@ -68,14 +68,14 @@ cudaError_t launch_multi_k(MultiStepArgs<T>& m, bool if_fits, bool* fits, bool p
     constexpr int V = Vec<T>::V, GPB = kBlock / G, TN = G * V;
     static std::atomic<int> shape[kShapeDevices];  // static storage: starts at 0
     int sms = 0, per_sm = 0;
-    const cudaError_t e = launch_shape(shape, k_step_multi<T, G, B, CHECK, PRIMAL>, long_smem<T, G>(1, kSegPer<G>), &sms,
+    const cudaError_t e = launch_shape(shape, k_step_multi<T, G, B, CHECK, PRIMAL>, long_smem<T, G>(1, kSegPer<T, G>), &sms,
                                        &per_sm);
     if (e != cudaSuccess) return e;
     int smem = 0, nlb[kMaxParts], need[kMaxParts], tiles[kMaxParts];
     for (int p = 0; p < m.nparts; ++p) {
         StepArgs<T>& a = m.part[p];
         a.pdl = pdl ? 1 : 0;
-        a.per = long_per<G>(a.n_lseg, sms);
+        a.per = long_per<T, G>(a.n_lseg, sms);
         nlb[p] = (a.n_lseg + a.per - 1) / a.per;
         smem = std::max(smem, long_smem<T, G>(a.n_lseg, a.per));
         need[p] = (a.n_short + GPB - 1) / GPB;

@@ -363,10 +363,15 @@ __device__ __forceinline__ bool long_row_reduce(T (&acc)[V], T* red) {
 // segments) 5.0 and 4.4 ms a pass of 256 iterations (3.5 with the short rows
 // in their own order), 8 LPs 4.1 and 3.7; on 100k x 200k with 50 long rows (200
 // segments), 2 LPs, 6.05 and 6.4.
-template <int G> constexpr int kSegPer = G <= 2 ? 4 / G : 1;
-template <int G>
+// Not in FP64, whose blocks are bound by their SM's FP64 pipe: few large ones,
+// started as the previous step's blocks leave room (programmatic dependent
+// launch), pile up on some SMs (1 and 2 LPs on the 20k x 50k matrix, 84 us an
+// iteration with four segments a block, 58 with one).
+template <typename T, int G>
+constexpr int kSegPer = std::is_same<T, double>::value || G > 2 ? 1 : 4 / G;
+template <typename T, int G>
 int long_per(int segments, int sms) {
-    return kSegPer<G> > 1 && segments > 4 * sms ? kSegPer<G> : 1;
+    return kSegPer<T, G> > 1 && segments > 4 * sms ? kSegPer<T, G> : 1;
 }
 // Dynamic shared memory of a long-row block: its partial sums, a vector per
 // lane, before them (wider rows than two lanes and narrower than 32) its
@@ -633,7 +638,7 @@ __device__ __forceinline__ void step_body(const StepArgs<T>& a, const int bx, co
     const bool active = col0 < a.ncol;
     const unsigned gmask = G == 32 ? 0xffffffffu : (((1u << G) - 1u) << ((threadIdx.x & 31) & ~(G - 1)));
     const char* const src = reinterpret_cast<const char*>(a.src + (active ? col0 : tile0));
-    const int per = kSegPer<G> > 1 ? a.per : 1, nlb = (a.n_lseg + per - 1) / per;
+    const int per = kSegPer<T, G> > 1 ? a.per : 1, nlb = (a.n_lseg + per - 1) / per;
     if (bx < nlb) {
         const int st = kBlock / per, sub = threadIdx.x / st, is = bx * per + sub;  // threads of a segment
         const bool some = is < a.n_lseg;
@@ -644,8 +649,8 @@ __device__ __forceinline__ void step_body(const StepArgs<T>& a, const int bx, co
         T acc[V];
 #pragma unroll
         for (int v = 0; v < V; ++v) acc[v] = T(0);
-        if (kSegPer<G> > 1 && per > 1) {
-            constexpr int SP = kSegPer<G>, ST = kBlock / SP;
+        if (kSegPer<T, G> > 1 && per > 1) {
+            constexpr int SP = kSegPer<T, G>, ST = kBlock / SP;
             // a row group takes SP pieces, next to one another, of at most E
             // entries; their columns and values come before the wait
             constexpr int E = (kStepSeg + GPB - 1) / GPB, PC = B / E < 1 ? 1 : B / E < SP ? B / E : SP;
