@@ -337,6 +337,7 @@ struct StepArgs {
     int t, ce;
     int uni;          // the group of every active column, or -1 if they belong to several
     int pdl;          // launched as a programmatic dependent of the previous step kernel
+    int hold;         // the next step kernel's blocks start when this grid has ended
     int hbm;          // the gathered block exceeds half of L2: the iterates come from HBM
 };
 
@@ -529,10 +530,11 @@ __device__ __forceinline__ void dual_epilogue(const StepArgs<T>& a, const TilePa
 // write those, and is launched without the attribute (launch_iteration).
 // Then let the next step kernel start its own prologue on the SMs this grid
 // frees.
-__device__ __forceinline__ void pdl_wait(int pdl) {
+// (hold: not before this grid ends, see early_release.)
+__device__ __forceinline__ void pdl_wait(int pdl, int hold) {
     if (pdl) {
         asm volatile("griddepcontrol.wait;" ::: "memory");
-        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+        if (!hold) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     }
 }
 
@@ -668,7 +670,7 @@ __device__ __forceinline__ void step_body(const StepArgs<T>& a, const int bx, co
                     w[p][j] = in ? ldg1(a.va + e) : T(0);
                 }
             __syncthreads();
-            pdl_wait(a.pdl);
+            pdl_wait(a.pdl, a.hold);
 #pragma unroll
             for (int p0 = 0; p0 < SP; p0 += PC) {
                 T xs[PC][E][V];
@@ -717,12 +719,12 @@ __device__ __forceinline__ void step_body(const StepArgs<T>& a, const int bx, co
                     va[q] = ldg1(a.va + rb + q);
                 }
                 __syncthreads();
-                pdl_wait(a.pdl);
+                pdl_wait(a.pdl, a.hold);
                 gather_held<T, V, G, B>(ci, va, src, pitch, beg - rb, end - rb, acc);
                 __syncthreads();
             } else {
                 __syncthreads();
-                pdl_wait(a.pdl);
+                pdl_wait(a.pdl, a.hold);
                 gather_range<T, V, G, B>(a.ci, a.va, src, pitch, beg, end, acc);
             }
             fin<V>(acc);
@@ -765,7 +767,7 @@ __device__ __forceinline__ void step_body(const StepArgs<T>& a, const int bx, co
     int4 rec = make_int4(0, 0, 0, 0);
     if (i < a.n_short) rec = __ldg(a.srec + i);
     __syncthreads();
-    pdl_wait(a.pdl);
+    pdl_wait(a.pdl, a.hold);
 #pragma unroll 1
     for (; i < a.n_short; i += stride) {
         const int row = rec.x, first = rec.y, pairs = rec.z, place = rec.w;
@@ -872,6 +874,18 @@ inline cudaError_t l2_bytes(long long* out) {
     return cudaSuccess;
 }
 
+// Whether a step lets the next step's blocks start before its own have ended.
+// They start wherever there is room, and where long-row blocks, the largest,
+// do, the FP64 pipes of some SMs get most of them.  At one and two lanes what
+// the early start saves still counts for more.  Microseconds an iteration, FP64,
+// long rows, with the early start and without: 8 LPs on 5k x 10k 21.7 and 19.5,
+// on 20k x 50k 50.1 and 45.2, 32 LPs on 3k x 6k 24.6 and 22.9; 4 LPs on 5k x 10k
+// 18.2 and 21.4; without long rows, 8 LPs on 20k x 20k 24.2 and 24.7.
+template <typename T>
+bool early_release(int lanes, bool long_rows) {
+    return !std::is_same<T, double>::value || lanes < 4 || !long_rows;
+}
+
 // Whether a step takes the short rows in their own order (Csr::nrec) and not
 // by length (Csr::srec); own: the bytes of the rows' two own blocks.  By
 // length, a warp's row groups run about as many entries each, but the rows'
@@ -905,6 +919,7 @@ StepArgs<T> step_args(bool primal, const IterData<T>& d, const IterBufs<T>& b, i
     a.ci = c.ci;
     a.va = primal ? d.at_vals : d.a_vals;
     const int lanes = row_group_lanes<T>(ncol, c.g_shift);
+    a.hold = !early_release<T>(lanes, d.A.n_long > 0 || d.At.n_long > 0);
     const long long own = 2LL * c.rows * ld * (long long)sizeof(T);
     a.srec = natural_order<T>(lanes, primal, own, l2) ? c.nrec : c.srec;
     a.pci = c.pci;
