@@ -168,45 +168,9 @@ __device__ __forceinline__ void ld_iterate(const char* src, unsigned c, unsigned
 // batch size).
 template <int G> constexpr int kRound = G >= 8 ? G : 8;
 
-// acc += entries [beg, end) of a row, in order, every lane of the row group
-// at the same ones (one broadcast load each); the gathers of B entries are
-// issued together.
-template <typename T, int V, int G, int B>
-__device__ __forceinline__ void gather_range(const int* __restrict__ ci, const T* __restrict__ va, const char* src,
-                                             unsigned pitch, int beg, int end, T (&acc)[V]) {
-    int e = beg;
-#pragma unroll 1
-    for (; e + B <= end; e += B) {
-        T w[B], xs[B][V];
-#pragma unroll
-        for (int j = 0; j < B; ++j) {
-            const unsigned c = (unsigned)__ldg(ci + e + j);
-            w[j] = ldg1(va + e + j);
-            ld_iterate(src, c, pitch, xs[j]);
-        }
-#pragma unroll
-        for (int j = 0; j < B; ++j)
-#pragma unroll
-            for (int v = 0; v < V; ++v) acc[v] = dot_acc(w[j], xs[j][v], acc[v]);
-    }
-    if (e < end) {
-        T w[B], xs[B][V];
-        const int first = beg + (e - beg) / kRound<G> * kRound<G>;
-#pragma unroll
-        for (int j = 0; j < B; ++j) {
-            const bool in = e + j < end;
-            const unsigned c = (unsigned)__ldg(ci + (in ? e + j : first));
-            w[j] = in ? ldg1(va + e + j) : T(0);
-            ld_iterate(src, c, pitch, xs[j]);
-        }
-#pragma unroll
-        for (int j = 0; j < B; ++j)
-#pragma unroll
-            for (int v = 0; v < V; ++v) acc[v] = dot_acc(w[j], xs[j][v], acc[v]);
-    }
-}
-
-// the same from shared memory
+// acc += entries [beg, end) of a long row, in order, from shared memory; every
+// lane of the row group is at the same ones, and the gathers of B entries are
+// issued together
 template <typename T, int V, int G, int B>
 __device__ __forceinline__ void gather_held(const int* ci, const T* va, const char* src, unsigned pitch, int beg,
                                             int end, T (&acc)[V]) {
@@ -375,12 +339,11 @@ int long_per(int segments, int sms) {
     return kSegPer<T, G> > 1 && segments > 4 * sms ? kSegPer<T, G> : 1;
 }
 // Dynamic shared memory of a long-row block: its partial sums, a vector per
-// lane, before them (wider rows than two lanes and narrower than 32) its
-// entries.  None where the matrix has no long row: L1 keeps what is not taken.
+// lane, before them (a block of one segment) its entries.  None where the matrix has no long row: L1 keeps what is not taken.
 template <typename T, int G>
 int long_smem(int segments, int per) {
     if (segments == 0) return 0;
-    const int sums = per * kBlock * 16, entries = G < 32 && per == 1 ? kStepSeg * (int)(sizeof(int) + sizeof(T)) : 0;
+    const int sums = per * kBlock * 16, entries = per == 1 ? kStepSeg * (int)(sizeof(int) + sizeof(T)) : 0;
     return sums > entries ? sums : entries;
 }
 
@@ -574,10 +537,10 @@ __device__ __forceinline__ dfloat add(dfloat a, dfloat b) { return a + b; }
 //   result does not depend on which block ends last.
 //   What bounds a long row is its block's chain of round trips, so the chain is
 //   short: one record (LongSeg) where there were four dependent loads, and
-//   below 32 lanes the entries are in shared memory or registers before the
-//   wait (64 LPs on the 20k x 50k power-law matrix, 256 iterations: 6.45 to
-//   6.28 ms a pass; at 32 lanes, whose blocks run in many waves, the detour
-//   cost 1.6%: 101 LPs on 200k x 400k 25.8 against 26.2 ms).
+//   the entries are in shared memory or registers before the wait (64 LPs on
+//   the 20k x 50k power-law matrix, 256 iterations: 6.45 to 6.28 ms a pass; at
+//   32 lanes, 100 LPs, microseconds an iteration: on 3k x 6k 17.5 to 16.8, on
+//   200k x 400k 379 to 375, on 1M x 2M 1823 to 1807).
 //   The other blocks: persistent over the short rows (srec), row group
 //   g taking records g, g + stride, ...; a warp's row groups take rows of
 //   about the same length (build_short_rows).
@@ -710,23 +673,17 @@ __device__ __forceinline__ void step_body(const StepArgs<T>& a, const int bx, co
                 for (int v = 0; v < V; ++v) acc[v] += part[(g * G + lane) * V + v];
         } else {
             const int beg = min(re, rb + grp * piece), end = min(re, beg + piece);
-            if constexpr (G < 32) {
-                // the segment's entries before the wait
-                T* const va = reinterpret_cast<T*>(red);
-                int* const ci = reinterpret_cast<int*>(va + kStepSeg);
-                for (int q = threadIdx.x; q < re - rb; q += kBlock) {
-                    ci[q] = __ldg(a.ci + rb + q);
-                    va[q] = ldg1(a.va + rb + q);
-                }
-                __syncthreads();
-                pdl_wait(a.pdl, a.hold);
-                gather_held<T, V, G, B>(ci, va, src, pitch, beg - rb, end - rb, acc);
-                __syncthreads();
-            } else {
-                __syncthreads();
-                pdl_wait(a.pdl, a.hold);
-                gather_range<T, V, G, B>(a.ci, a.va, src, pitch, beg, end, acc);
+            // the segment's entries before the wait
+            T* const va = reinterpret_cast<T*>(red);
+            int* const ci = reinterpret_cast<int*>(va + kStepSeg);
+            for (int q = threadIdx.x; q < re - rb; q += kBlock) {
+                ci[q] = __ldg(a.ci + rb + q);
+                va[q] = ldg1(a.va + rb + q);
             }
+            __syncthreads();
+            pdl_wait(a.pdl, a.hold);
+            gather_held<T, V, G, B>(ci, va, src, pitch, beg - rb, end - rb, acc);
+            __syncthreads();
             fin<V>(acc);
             if (!long_row_reduce<T, V, G>(acc, reinterpret_cast<T*>(red))) return;
         }
