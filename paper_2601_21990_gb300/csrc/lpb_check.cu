@@ -770,6 +770,19 @@ __global__ void __launch_bounds__(256) k_extract_tiles(int n, int m, int ld, con
     }
 }
 
+// zeros for the points of the LPs that are done (launch_zero_points)
+__global__ void __launch_bounds__(256) k_zero_points(const ColRecord* __restrict__ rec, int count, int n, int m,
+                                                     double* __restrict__ x, double* __restrict__ y) {
+    for (int q = blockIdx.y; q < count; q += gridDim.y) {
+        if (rec[q].status < 0) continue;
+        const int stride = gridDim.x * blockDim.x;
+        if (x)
+            for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) x[(size_t)q * n + i] = 0.0;
+        if (y)
+            for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < m; i += stride) y[(size_t)q * m + i] = 0.0;
+    }
+}
+
 // moves column src[p] -> dst[p] in every row of the state blocks (the
 // primal reflected point Xbar and anchor X0, the dual iterate and anchor)
 template <typename T>
@@ -1385,6 +1398,15 @@ cudaError_t launch_admit(const CheckData& d, const IterData<T>& it, const IterBu
     if (e != cudaSuccess) return e;
     k_init_iterates<T><<<blocks_for((size_t)(d.n + d.m) * count, 256), 256, 0, s>>>(a, b.Xbar, b.X0, b.Y, b.Y0, warm_x,
                                                                                     warm_y, wsx, wsy);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_zero_points(const ColRecord* rec, int count, int n, int m, double* x, double* y, cudaStream_t s) {
+    if (count <= 0) return cudaSuccess;
+    // most LPs' blocks leave at once: no more of them than fill the GPU a few times
+    const int rows = n > m ? n : m, each = count < 128 ? 64 : count < 8192 ? 8192 / count : 1;
+    const dim3 grid(blocks_for(rows, 256, each), count < 65535 ? count : 65535);
+    k_zero_points<<<grid, 256, 0, s>>>(rec, count, n, m, x, y);
     return cudaGetLastError();
 }
 

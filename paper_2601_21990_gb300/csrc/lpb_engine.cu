@@ -436,12 +436,12 @@ lpb_err lane_admit(lpb_ctx* h, Lane& ln, GroupRun& g, const lpb_lp_spec* specs_d
         if (rc.status >= 0) {
             set_result(g.res[q], rc, rc.status, 0, 0);
             gone.push_back(c0 + q);
-            // every other LP's point is extracted; this one has none: zeros
-            if (g.x_dev) LPB_CU(cudaMemsetAsync(g.x_dev + (size_t)q * h->n, 0, sizeof(double) * h->n, s));
-            if (g.y_dev && h->m > 0)
-                LPB_CU(cudaMemsetAsync(g.y_dev + (size_t)q * h->m, 0, sizeof(double) * h->m, s));
         }
     }
+    // every other LP's point is extracted; these have none: zeros (one launch,
+    // where two memsets for each took 2.6 us apiece)
+    if (!gone.empty() && (g.x_dev || g.y_dev))
+        LPB_CU(launch_zero_points(ln.rec + c0, count, h->n, h->m, g.x_dev, g.y_dev, s));
     g.live -= (int)gone.size();
     lpb_err rc = compact<T>(h, ln, gone, s, nullptr);
     if (rc != LPB_OK) return rc;

@@ -337,6 +337,10 @@ cudaError_t launch_extract(const CheckData& d, const IterBufs<T>& b, int ld, con
                            double* const* outp_dev, int count, const double* xl_base, const double* xu_base,
                            cudaStream_t s);
 
+// Zeros for the points (x + q n, y + q m; either may be null) of the LPs q of
+// rec[0 .. count) that are done (status >= 0).
+cudaError_t launch_zero_points(const ColRecord* rec, int count, int n, int m, double* x, double* y, cudaStream_t s);
+
 // Moves columns sc_dev[p] of an FP32 lane to columns dc_dev[p] of a polish
 // lane in precision TD (double or dfloat): the iterates and anchors widened,
 // the per-column data copied, the TD parameters rebuilt from the FP64

@@ -16,6 +16,7 @@ struct State {
     std::map<const void*, std::string> names;  // kernels, by host function
     std::map<std::string, long> launched;
     std::map<void*, size_t> live;              // device allocations
+    long memsets = 0;
     long waits = 0;                             // cudaMalloc and cudaFree
     long fail_from = 0, fail_to = 0;           // device allocations [fail_from, fail_to) from now on fail (1: the next)
     cudaError_t last = cudaSuccess;
@@ -50,6 +51,10 @@ long launches(const char* part) {
 bool last_error() {
     Lock l(st().mu);
     return st().last != cudaSuccess;
+}
+long memsets() {
+    Lock l(st().mu);
+    return st().memsets;
 }
 std::function<void(void*, size_t)> on_read;
 
@@ -140,6 +145,10 @@ cudaError_t cudaMemcpy(void* d, const void* s, size_t n, cudaMemcpyKind k) {
 }
 cudaError_t cudaMemcpyAsync(void* d, const void* s, size_t n, cudaMemcpyKind k, cudaStream_t) { return cudaMemcpy(d, s, n, k); }
 cudaError_t cudaMemset(void* d, int v, size_t n) {
+    {
+        fake::Lock l(fake::st().mu);
+        ++fake::st().memsets;
+    }
     if (n) std::memset(d, v, n);
     return cudaSuccess;
 }

@@ -23,6 +23,8 @@ bool last_error();
 // calls so far that wait for the whole device: cudaMalloc and cudaFree
 long device_waits();
 
+// calls so far of cudaMemset and cudaMemsetAsync
+long memsets();
 // called after each copy from the device, with its destination and bytes (set
 // it while no other thread copies)
 extern std::function<void(void*, size_t)> on_read;

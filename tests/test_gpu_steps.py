@@ -305,3 +305,33 @@ def test_row_orders_agree_on_a_large_matrix(lpb, lps, lanes):
             assert np.array_equal(a, b), q
     wide.free(), narrow.free()
     h.close()
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("lps", [1, 5, 200, 1500])
+def test_points_of_empty_boxes_are_zero_among_others(lpb, precision, lps):
+    """LPs whose box is empty end at admission, with zeros for their points;
+    the others' points are those of the same LPs without them.  One check, so
+    no restart couples the LPs."""
+    lp = _lp(40, 300, 6, 3)
+    sp = _specs(lp, lps, lps)
+    sp.kind = np.where(np.arange(lps) % 3 == 0, 1, sp.kind)
+    empty = np.arange(lps) % 3 == 0
+    sp.lo, sp.hi = np.where(empty, 5.0, sp.lo), np.where(empty, 4.0, sp.hi)
+    specs = lpb.specs_array(sp.kind, sp.var, sp.lo, sp.hi, sp.sign)
+    h = lpb.Handle(lp, precision=lpb.FP64 if precision == "fp64" else lpb.MIXED)
+    junk = h.solve(lpb.specs_array(np.zeros(lps, int), sp.var), tol=1e-12, max_iter=64)  # (memory with points in it)
+    junk.free()
+    b = h.solve(specs, tol=1e-12, max_iter=64)
+    assert (b.results()["status"][empty] == lpb.PRIMAL_INFEASIBLE).all()
+    rest = np.flatnonzero(~empty)
+    alone = h.solve(specs[rest], tol=1e-12, max_iter=64) if rest.size else None
+    for q in range(lps):
+        _, x, y = b.result(q)
+        if empty[q]:
+            assert not x.any() and not y.any(), q
+        else:
+            _, x1, y1 = alone.result(int(np.searchsorted(rest, q)))
+            assert np.array_equal(x, x1) and np.array_equal(y, y1), q
+    b.free()
+    h.close()

@@ -1,4 +1,5 @@
-"""CPU: the library's host code where device memory runs short.  The
+"""CPU: the library's host code where device memory runs short, and what it asks
+of the runtime.  The
 library's objects are linked with a stand-in for the CUDA runtime
 (tests/native/fake_cuda.cpp) that needs no GPU and fails allocations on demand."""
 import os
@@ -46,3 +47,7 @@ def test_a_layout_without_memory_leaves_the_step_kernels(objects, tmp_path):
 
 def test_a_servers_budget_covers_layouts_and_requests_come_first(objects, tmp_path):
     _run(objects, tmp_path, "serve_layout_test")
+
+
+def test_admission_takes_as_many_calls_for_any_number_of_infeasible_lps(objects, tmp_path):
+    _run(objects, tmp_path, "admit_calls_test")
