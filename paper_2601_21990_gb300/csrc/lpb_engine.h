@@ -206,6 +206,9 @@ cudaError_t launch_resident(const IterPart<T>* parts, ResPlan* const* plans, int
 // keep_stream: once the handle's stream has come to this point, without a wait
 // for the device; launches queued on that stream may use them.
 void free_res_plans(lpb_ctx* h, bool keep_stream = false);
+// From now on `account` is asked and told (lpb_ctx::res_charge; empty: none).
+// The layouts that are there belong to the handle, on no account.
+void set_res_account(lpb_ctx* h, std::function<bool(int64_t)> account);
 // first free run of count residual slots, or -1
 int lane_find_slots(const Lane& ln, int count);
 // a free group id, or -1

@@ -33,6 +33,7 @@
 #include <cstring>
 #include <memory>
 #include <new>
+#include <utility>
 
 #include "lpb_engine.h"
 #include "lpb_resident.h"
@@ -597,6 +598,11 @@ cudaError_t res_launch(const ResArgs<T>& g, int threads, size_t smem, cudaStream
 }
 
 }  // namespace
+
+void set_res_account(lpb_ctx* h, std::function<bool(int64_t)> account) {
+    h->res_charge = std::move(account);
+    for (ResPlan* p : h->res_plans) p->charged = 0;
+}
 
 void free_res_plans(lpb_ctx* h, bool keep_stream) {
     if (!h->res_plans.empty()) h->ws_epoch += 1;  // captured intervals hold them

@@ -514,7 +514,7 @@ lpb_err lpb_server_attach(lpb_server_t srv, lpb_handle h, int32_t* matrix_id) {
     }
     *matrix_id = (int32_t)srv->mats.size();
     Matrix* mp = M.get();
-    h->res_charge = [srv](int64_t bytes) { return charge_layout(srv, bytes); };
+    set_res_account(h, [srv](int64_t bytes) { return charge_layout(srv, bytes); });
     srv->mats.push_back(std::move(M));
     srv->st.hbm_used_bytes = srv->used;
     srv->workers.emplace_back(worker_main, srv, mp, (int)*matrix_id);
@@ -705,7 +705,7 @@ void lpb_server_destroy(lpb_server_t srv) {
     cudaSetDevice(srv->device);
     for (auto& mp : srv->mats) {
         if (mp->h && mp->h->stream) cudaStreamSynchronize(mp->h->stream);
-        if (mp->h) mp->h->res_charge = nullptr;
+        if (mp->h) set_res_account(mp->h, {});
         lane_free(mp->lane32);
         lane_free(mp->lanep);
     }

@@ -108,6 +108,12 @@ int main() {
         if (used(s) > o.hbm_budget_bytes) return fail_at("over budget", used(s));
         lpb_server_destroy(s);
         if (h->res_charge) return fail_at("the account outlives its server", round);
+        // a layout made for one server is not on the next one's account
+        o.hbm_budget_bytes = (int64_t)1 << 34;
+        if (lpb_server_create(&o, &s) != LPB_OK || lpb_server_attach(s, h, &id) != LPB_OK) return fail_at("second server", round);
+        lpb_tuning t{64, 64, 0, 0};
+        if (lpb_set_tuning(h, &t) != LPB_OK || used(s) != lanes) return fail_at("account of the second server", used(s) - lanes);
+        lpb_server_destroy(s);
         lpb_destroy(h);
         if (fake::live_bytes() != 0) return fail_at("memory left", (long long)fake::live_bytes());
     }
