@@ -75,6 +75,7 @@ struct Csr {
     float* v32lo = nullptr;     // v64 - v32 rounded to FP32: (v32, v32lo) is v64 in double-float
     int* long_rows = nullptr;   // rows with > long_thr entries
     int n_long = 0;
+    long long long_nnz = 0;     // their entries
     // The other rows as the step kernels take them (build_short_rows): each
     // row's entries together, from a multiple of four on, in windows of rows
     // sorted by length, and its cost and bounds at its record's place.

@@ -802,6 +802,7 @@ static cudaError_t build_long_segments(Csr& a, cudaStream_t s) {
     std::vector<int> part0(a.n_long + 1, 0);
     int most = 0;
     for (int i = 0; i < a.n_long; ++i) {
+        a.long_nnz += rows[i].z - rows[i].y;
         const int segs = std::max(1, (rows[i].z - rows[i].y + kStepSeg - 1) / kStepSeg);
         part0[i + 1] = part0[i] + segs;
         most = std::max(most, segs);
@@ -827,6 +828,7 @@ void free_long_rows(Csr& a) {
     a.long_rows = nullptr;
     a.lseg = nullptr;
     a.n_long = a.n_lseg = 0;
+    a.long_nnz = 0;
 }
 
 cudaError_t build_long_rows(Csr& a, cudaStream_t s) {
@@ -836,6 +838,7 @@ cudaError_t build_long_rows(Csr& a, cudaStream_t s) {
         free_long_rows(a);
     }
     a.n_long = 0;
+    a.long_nnz = 0;
     a.n_lseg = 0;
     if (a.rows == 0) return cudaSuccess;
     StreamMem mem(s);
@@ -857,8 +860,7 @@ cudaError_t build_long_rows(Csr& a, cudaStream_t s) {
 }
 
 void free_short_rows(Csr& a) {
-    if (a.srec) cudaFree(a.srec);  // with the rows' vectors behind it
-    if (a.pci) cudaFree(a.pci);    // with the values behind it
+    if (a.srec) cudaFree(a.srec);  // with all that lies behind it
     a.srec = a.nrec = nullptr;
     a.pci = nullptr;
     a.pv32 = a.pk32 = nullptr;
@@ -881,28 +883,42 @@ cudaError_t build_short_rows(Csr& a, RowVectors<float> v32, RowVectors<double> v
     free_short_rows(a);
     const int n = a.rows - a.n_long;
     if (n <= 0) return cudaSuccess;
-    // the records and the rows' vectors
+    // one allocation: the records, the rows' vectors, and the entries, at most
+    // three a row more than the short rows have (their exact number would cost
+    // a wait); the long rows' entries stay where they are
+    const size_t entries = (size_t)(a.nnz - a.long_nnz) + 3 * (size_t)n;
     size_t bytes = 0;
     auto take = [&](bool wanted, size_t size) {
         const size_t at = bytes;
         if (wanted) bytes += (size + 255) / 256 * 256;
         return at;
     };
-    const size_t at_rec = take(true, sizeof(int4) * n), at_nrec = take(true, sizeof(int4) * n);
-    const size_t at_k32 = take(v32.vals, 16 * (size_t)n), at_k64 = take(v64.vals, 32 * (size_t)n);
-    const size_t at_kdf = take(vdf.vals, 32 * (size_t)n);
+    const size_t at_rec = take(true, sizeof(int4) * n), at_nrec = take(true, sizeof(int4) * n), at_ci = take(true, 4 * entries);
+    const size_t at_v32 = take(v32.vals, 4 * entries), at_k32 = take(v32.vals, 16 * (size_t)n);
+    const size_t at_v64 = take(v64.vals, 8 * entries), at_k64 = take(v64.vals, 32 * (size_t)n);
+    const size_t at_vdf = take(vdf.vals, 8 * entries), at_kdf = take(vdf.vals, 32 * (size_t)n);
     char* mem = nullptr;
     if ((e = cudaMalloc((void**)&mem, bytes)) != cudaSuccess) return e;
     a.srec = (int4*)(mem + at_rec);
     a.nrec = (int4*)(mem + at_nrec);
-    if (v32.vals) a.pk32 = (float*)(mem + at_k32);
-    if (v64.vals) a.pk64 = (double*)(mem + at_k64);
-    if (vdf.vals) a.pkdf = (dfloat*)(mem + at_kdf);
+    a.pci = (int*)(mem + at_ci);
+    if (v32.vals) {
+        a.pv32 = (float*)(mem + at_v32);
+        a.pk32 = (float*)(mem + at_k32);
+    }
+    if (v64.vals) {
+        a.pv64 = (double*)(mem + at_v64);
+        a.pk64 = (double*)(mem + at_k64);
+    }
+    if (vdf.vals) {
+        a.pvdf = (dfloat*)(mem + at_vdf);
+        a.pkdf = (dfloat*)(mem + at_kdf);
+    }
     const int windows = (a.rows + kWindow - 1) / kWindow;
     const size_t most = std::max((size_t)a.rows, (size_t)n);
     StreamMem scratch(s);
-    if ((e = scratch.take(sizeof(int) * (most * 2 + 1))) != cudaSuccess) return e;
-    int *cnt = (int*)scratch.p, *first = cnt + most, *total = first + most;
+    if ((e = scratch.take(sizeof(int) * most * 2)) != cudaSuccess) return e;
+    int *cnt = (int*)scratch.p, *first = cnt + most;
     k_short_count<<<windows, 256, 0, s>>>(a.rp, a.rows, a.long_thr, cnt);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if ((e = exclusive_scan_i32(cnt, first, windows, nullptr, s)) != cudaSuccess) return e;
@@ -910,9 +926,7 @@ cudaError_t build_short_rows(Csr& a, RowVectors<float> v32, RowVectors<double> v
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     k_short_fours<<<grid_for(n, 256), 256, 0, s>>>(a.srec, n, cnt);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    if ((e = exclusive_scan_i32(cnt, first, n, total, s)) != cudaSuccess) return e;
-    int fours = 0;
-    if ((e = cudaMemcpyAsync(&fours, total, sizeof(int), cudaMemcpyDeviceToHost, s)) != cudaSuccess) return e;
+    if ((e = exclusive_scan_i32(cnt, first, n, nullptr, s)) != cudaSuccess) return e;
     k_short_place<<<grid_for(n, 256), 256, 0, s>>>(a.srec, n, first);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     k_short_flags<<<grid_for(a.rows, 256), 256, 0, s>>>(a.rp, a.rows, a.long_thr, cnt);
@@ -922,18 +936,6 @@ cudaError_t build_short_rows(Csr& a, RowVectors<float> v32, RowVectors<double> v
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     k_short_narrow<<<grid_for(a.rows, 256), 256, 0, s>>>(a.srec, cnt, a.rp, a.rows, a.long_thr, first, a.nrec);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    // the entries: as many as the short rows have, the long rows' stay where they are
-    if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return e;
-    const size_t entries = 4 * (size_t)fours;
-    bytes = 0;
-    take(true, 4 * entries);
-    const size_t at_v32 = take(v32.vals, 4 * entries), at_v64 = take(v64.vals, 8 * entries);
-    const size_t at_vdf = take(vdf.vals, 8 * entries);
-    if ((e = cudaMalloc((void**)&mem, bytes ? bytes : 1)) != cudaSuccess) return e;
-    a.pci = (int*)mem;
-    if (v32.vals) a.pv32 = (float*)(mem + at_v32);
-    if (v64.vals) a.pv64 = (double*)(mem + at_v64);
-    if (vdf.vals) a.pvdf = (dfloat*)(mem + at_vdf);
     k_short_cols<<<grid_for((long long)n * 32, 256, kStatCap), 256, 0, s>>>(a.srec, n, a.rp, a.ci, a.pci);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if ((e = pack_vals<float>(a, n, v32, a.pv32, a.pk32, s)) != cudaSuccess) return e;
